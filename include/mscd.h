@@ -86,7 +86,7 @@ typedef struct mscd_params {
     int32_t blocks_per_sm;   /* first class: CTAs per SM (0 = from occupancy)           */
     int32_t mid_slots;       /* node slots of an optional second shared-memory class
                                 (power of 2 >= 32; 0 = none)                            */
-    int32_t global_warps_per_sm; /* global-arena classes: resident units per SM (16)     */
+    int32_t global_warps_per_sm; /* global-arena classes: resident units per SM (24)     */
     int32_t global_slots;    /* node slots of the first global-arena class (power of 2;
                                 0 = 8 times the last shared-memory class)                */
     int64_t max_rounds;      /* grow/prune repetitions per unit before ETIMEOUT (1e6)     */
@@ -96,9 +96,9 @@ typedef struct mscd_params {
                                 one launch per scale and slot class, one unit per warp,
                                 statically mapped (no persistence, no work stealing); the
                                 results are identical, only the speed differs           */
-    int32_t hash_smem_slots; /* global-arena classes of at most this many slots keep
-                                their hash table (and group bounds) in shared memory,
-                                the slot arrays in the arena (0 = none)               */
+    int32_t hash_smem_slots; /* classes after the shared-memory ones of at most this
+                                many slots run in shared memory too, where one unit's
+                                state fits it (0 = none)                              */
     int32_t list_hash_bits;  /* testing only: keep this many low bits (1..63) of each
                                 member list's 64-bit hash, so that different lists
                                 share hashes and dedup's exact comparison and

@@ -290,7 +290,7 @@ int mscd_create(mscd_ctx **out, int device, const mscd_params *params) {
     if (c->p.max_rounds <= 0) c->p.max_rounds = 1000000;
     if (c->p.smem_slots < 0) c->p.smem_slots = 0;
     if (c->p.mid_slots < 0) c->p.mid_slots = 0;
-    if (c->p.global_warps_per_sm <= 0) c->p.global_warps_per_sm = 16;
+    if (c->p.global_warps_per_sm <= 0) c->p.global_warps_per_sm = GLOBAL_MIN_BLOCKS * GLOBAL_CTA_THREADS / 32;
     if (c->p.list_hash_bits < 0 || c->p.list_hash_bits > 63 || c->p.global_slots < 0 ||
         (c->p.global_slots & (c->p.global_slots - 1)) ||
         (c->p.schedule != MSCD_SCHED_PERSISTENT && c->p.schedule != MSCD_SCHED_PER_SCALE)) {

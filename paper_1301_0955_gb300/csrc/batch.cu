@@ -38,7 +38,7 @@ __global__ void shift_left(const i64 *src, i64 m, int s, i64 *dst) {
 // Same expression as the degree kernel of graph preparation.
 __global__ void log_degrees(const i64 *k, i64 m, float *logk) {
     for (i64 i = (i64)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (i64)gridDim.x * blockDim.x)
-        logk[i] = k[i] ? logf((float)k[i]) : 0.0f;
+        logk[i] = k[i] ? log2f((float)k[i]) : 0.0f;
 }
 
 unsigned grid_for(i64 m) { return (unsigned)std::max<i64>(1, std::min<i64>((m + 255) / 256, 152 * 8)); }

@@ -21,7 +21,7 @@ struct DevGraph {
     const i32 *col = nullptr;    // int32[nnz]
     const i64 *wfx = nullptr;    // int64[nnz] exact fixed-point weights, null = unweighted
     const i64 *k = nullptr;      // int64[n] weighted degree (weight units)
-    const float *logk = nullptr;   // float[n] logf(k) (0 where k = 0), for the binary32 priority keys
+    const float *logk = nullptr;   // float[n] log2f(k) (0 where k = 0), for the binary32 priority keys
     i64 kmax = 0;                  // largest k_u
     int unit_exp = 0;            // weight unit 2^unit_exp
     i64 volume = 0;              // sum of k

@@ -68,7 +68,7 @@ __device__ __forceinline__ dd mul_d(dd x, double y) {
     p.lo += x.lo * y;
     return fast_two_sum(p.hi, p.lo);
 }
-__device__ __noinline__ dd div(dd x, dd y) {
+static __device__ __noinline__ dd div(dd x, dd y) {
     double q1 = x.hi / y.hi;
     dd r = add(x, neg(mul_d(y, q1)));
     double q2 = r.hi / y.hi;
@@ -84,7 +84,7 @@ __device__ __forceinline__ dd from_i64(i64 a) {  // exact for |a| < 2^62
 
 // 2 atanh(z) = log((1+z)/(1-z)), |z| <= 1/3: odd power series, summed until
 // the term falls below 2^-112 of the sum.
-__device__ __noinline__ dd atanh2(dd z) {
+static __device__ __noinline__ dd atanh2(dd z) {
     dd z2 = mul(z, z);
     dd term = z, sum = z;
     for (int j = 1; j < 90; ++j) {
@@ -97,7 +97,7 @@ __device__ __noinline__ dd atanh2(dd z) {
 }
 
 // log(a1/a2) in double-double.
-__device__ __noinline__ dd log_ratio(i64 a1, i64 a2) {
+static __device__ __noinline__ dd log_ratio(i64 a1, i64 a2) {
     i64 diff = a1 - a2;
     u64 ad = diff < 0 ? (u64)(-diff) : (u64)diff;
     if (ad <= (u64)a2 / 2) {
@@ -147,7 +147,7 @@ __device__ __forceinline__ bool power_is(i64 base, u64 e, i64 target) {
     return acc == (unsigned __int128)target;
 }
 
-__device__ __noinline__ bool is_tie(i64 a1, i64 a2, i64 b1, i64 b2, double alpha) {
+static __device__ __noinline__ bool is_tie(i64 a1, i64 a2, i64 b1, i64 b2, double alpha) {
     i64 g = gcd64(a1, a2);
     i64 an = a1 / g, ad = a2 / g;
     g = gcd64(b1, b2);
@@ -188,7 +188,7 @@ __device__ __forceinline__ double log_ratio_fast(i64 a1, i64 a2) {
 // Stages 3 and 4.  The result is returned by value (the sign plus one, in
 // bits 0-1, and the EXACT_* flags above it) so that no caller state has its
 // address taken by this out-of-line function.
-__device__ __noinline__ u32 sign_slow(i64 a1, i64 a2, i64 b1, i64 b2, double alpha) {
+static __device__ __noinline__ u32 sign_slow(i64 a1, i64 a2, i64 b1, i64 b2, double alpha) {
     const u32 slow = EXACT_SLOW << 2;
     if (is_tie(a1, a2, b1, b2, alpha)) return slow | 1u;
     dd L1 = log_ratio(a1, a2), L2 = log_ratio(b1, b2);
@@ -244,33 +244,89 @@ __device__ __forceinline__ int sign_delta32(i64 a1, i64 a2, i64 b1, i64 b2, doub
     return sign_delta(a1, a2, b1, b2, alpha, flags);
 }
 
+// The add and remove tests where the cheap bounds below leave them open, and
+// the order of two near keys.  Out of line: these are rare (a few per cent of
+// the decisions), and inlined at every site the two log stages made most of
+// the kernel's code (a third of the stall cycles waited for instructions) and
+// of its registers.  The result comes back by value: the sign plus one in
+// bits 0-1, the EXACT_* flags above.
+static __device__ __noinline__ u32 sign_open(i64 a1, i64 a2, i64 b1, i64 b2, double alpha) {
+    u32 flags = 0;
+    const int s = sign_delta32(a1, a2, b1, b2, alpha, (float)alpha, flags);
+    return (flags << 2) | (u32)(s + 1);
+}
+
+// Sign of the ranking comparison log(dx/dy) - alpha log(kx/ky) where it takes
+// whole numbers only: alpha = 1 (dx ky against dy kx) and, for values below
+// 2^31, alpha = 1/2 (dx^2 ky against dy^2 kx).  At these two scales unweighted
+// graphs tie all the time, and the binary64 logarithms and the general tie
+// test of sign_delta cost some 10^4 cycles a pair here.  2: not such a case.
+__device__ __forceinline__ int sign_whole(i64 dx, i64 dy, i64 kx, i64 ky, double alpha) {
+    if (kx == ky) return (dx > dy) - (dx < dy);
+    if (dx == dy) return (ky > kx) - (ky < kx);
+    unsigned __int128 l, r;
+    if (alpha == 1.0) {
+        l = (unsigned __int128)(u64)dx * (u64)ky;
+        r = (unsigned __int128)(u64)dy * (u64)kx;
+    } else if (alpha == 0.5 && ((dx | dy | kx | ky) >> 31) == 0) {
+        l = (unsigned __int128)((u64)dx * (u64)dx) * (u64)ky;
+        r = (unsigned __int128)((u64)dy * (u64)dy) * (u64)kx;
+    } else {
+        return 2;
+    }
+    return (l > r) - (l < r);
+}
+
+// Node ia (d_in da, degree ka) ranks before node ib (db, kb): larger
+// 2d/k^alpha, equal ones by id.  Bit 0 the answer, EXACT_* flags above it.
+// The pair is always evaluated with the smaller id first, so both orders give
+// the same answer.
+static __device__ __noinline__ u32 ranks_near(i64 da, i64 ka, i32 ia, i64 db, i64 kb, i32 ib, double alpha) {
+    const bool swap = ia > ib;
+    const i64 dx = swap ? db : da, dy = swap ? da : db;
+    const i64 kx = swap ? kb : ka, ky = swap ? ka : kb;
+    u32 flags = 0;
+    int s = sign_whole(dx, dy, kx, ky, alpha);
+    if (s == 2) s = sign_delta(dx, dy, kx, ky, alpha, flags);
+    const bool xfirst = s >= 0;  // equal: the smaller id
+    return (flags << 1) | (u32)(swap != xfirst);
+}
+
 // Add test for a node outside c: (K+2d)/(V+k)^alpha > K/V^alpha.
-__device__ __forceinline__ bool add_test(i64 K, i64 V, i64 d, i64 k, double alpha, float alpha32, u32 &flags) {
+__device__ __forceinline__ bool add_test(i64 K, i64 V, i64 d, i64 k, double alpha, u32 &flags) {
     if (K == 0) return true;  // f_c = 0 < f_{c+n} because d > 0
-    return sign_delta32(K + 2 * d, K, V + k, V, alpha, alpha32, flags) > 0;
+    const u32 r = sign_open(K + 2 * d, K, V + k, V, alpha);
+    flags |= r >> 2;
+    return (r & 3u) == 2u;
 }
 
 // Remove test for a member: (K-2d)/(V-k)^alpha > K/V^alpha.
-__device__ __forceinline__ bool remove_test(i64 K, i64 V, i64 d, i64 k, double alpha, float alpha32, u32 &flags) {
+__device__ __forceinline__ bool remove_test(i64 K, i64 V, i64 d, i64 k, double alpha, u32 &flags) {
     if (K == 0 || K - 2 * d == 0) return false;  // f_{c\n} = 0 <= f_c
-    return sign_delta32(K - 2 * d, K, V - k, V, alpha, alpha32, flags) > 0;
+    const u32 r = sign_open(K - 2 * d, K, V - k, V, alpha);
+    flags |= r >> 2;
+    return (r & 3u) == 2u;
 }
 
-// Necessary conditions (cheap filters, no transcendental): log1p(x) <= x and
-// log1p(y) >= y/(1+y) give   add  => 2d(V+k) > alpha K k,
-//                            remove => 2d(V-k) < alpha K k.
-// Evaluated in binary32 (products stay below 2^125 < FLT_MAX); each side
-// carries at most ~6 roundings of 2^-24 (alpha32 included), so a 2^-19
-// margin keeps the filters one-sided.
-__device__ __forceinline__ bool add_possible(i64 K, i64 V, i64 d, i64 k, float alpha32) {
-    float lhs = 2.0f * i2f(d) * i2f(V + k);  // V + k formed exactly in int64
-    float rhs = alpha32 * i2f(K) * i2f(k);
-    return lhs > rhs * (1.0f - 0x1p-19f);
+// Bounds that settle most tests without a transcendental.  With x = 2d/K and
+// y = k/V,
+//   x(6+3x)/(6+6x+x^2) <= log1p(x) <= x(6+x)/(6+4x),   the same for y
+// (Pade approximants; the differences have derivatives of one sign for
+// positive arguments: x^4/((1+x)(6+6x+x^2)^2) and 4x^3/((1+x)(6+4x)^2)).
+// Each side is computed within 20 roundings of 2^-24 (the fast division within
+// 2 ulp); the margin 2^-18 covers both.
+__device__ __forceinline__ float log1p_low(float x) {
+    return __fdividef(x * fmaf(3.0f, x, 6.0f), fmaf(x, x + 6.0f, 6.0f));
 }
-__device__ __forceinline__ bool remove_possible(i64 K, i64 V, i64 d, i64 k, float alpha32) {
-    float lhs = 2.0f * i2f(d) * i2f(V - k);  // no cancellation: V - k exact in int64
-    float rhs = alpha32 * i2f(K) * i2f(k);
-    return lhs < rhs * (1.0f + 0x1p-19f);
+__device__ __forceinline__ float log1p_high(float x) { return __fdividef(x * (6.0f + x), fmaf(4.0f, x, 6.0f)); }
+
+// (K+2d)/(V+k)^alpha > K/V^alpha for certain.
+__device__ __forceinline__ bool raises(float K, float V, float d, float k, float alpha32) {
+    return log1p_low(__fdividef(2.0f * d, K)) > alpha32 * log1p_high(__fdividef(k, V)) * (1.0f + 0x1p-18f);
+}
+// (K+2d)/(V+k)^alpha < K/V^alpha for certain.
+__device__ __forceinline__ bool lowers(float K, float V, float d, float k, float alpha32) {
+    return log1p_high(__fdividef(2.0f * d, K)) < alpha32 * log1p_low(__fdividef(k, V)) * (1.0f - 0x1p-18f);
 }
 
 }  // namespace exact

@@ -139,7 +139,7 @@ __global__ void degrees(const i64 *rp, const i64 *wfx, i64 n, i64 *k, float *log
         }
         if (lane == 0) {
             k[u] = (i64)s;
-            logk[u] = s ? logf((float)(i64)s) : 0.0f;
+            logk[u] = s ? log2f((float)(i64)s) : 0.0f;
             tot += s;
             kmax = s > kmax ? s : kmax;
             tot_d += sd;

@@ -4,7 +4,15 @@
 #include "common.cuh"
 
 #define GROW_MAX_THREADS 512
-#define GLOBAL_CTA_THREADS 256  // threads per CTA of the global-arena classes
+#define GROW_SMEM_MAX (220 * 1024)  // dynamic shared memory of a CTA of a shared-memory class, at most
+// Global-arena classes: threads per CTA, and the CTAs an SM has registers for.
+// Up to 32,768 slots the loop's 80 registers let 24 units share an SM: on the
+// 1-of-80 weighted 1M-node run the 8,192-slot class takes 283 ms, 316 at 16
+// units (128 registers), 278 at 32 (64, spilling a little; slower than 24
+// where few units run).  The few units of the wider classes take 128.
+#define GLOBAL_CTA_THREADS 128
+#define GLOBAL_MIN_BLOCKS 6
+#define WIDE_MIN_BLOCKS 4
 
 struct GrowArgs {
     DevGraph G;
@@ -29,9 +37,9 @@ struct GrowArgs {
     // per-warp node-slot state
     int cap;                // node slots per unit (power of 2, >= 32)
     int use_smem;           // 1: dynamic shared memory, 0: global arena
-    int bounds_smem;        // global arena with the group bounds in dynamic shared memory
-    int hash_smem;          // ... and the hash table too (after the bounds)
-    size_t smem_per_warp;   // dynamic shared memory of one warp in a global-arena class
+    // global arena up to 32768 slots: dynamic shared memory of one warp, the group
+    // bounds (8 bytes per 32 slots)
+    size_t smem_per_warp;
     unsigned char *big_seed;  // per seed: outgrew this class at a finer scale (first class only; may be null)
     unsigned char *gstate;  // global arena (warps * state_bytes)
     size_t state_bytes;     // per warp
@@ -52,13 +60,14 @@ struct GrowArgs {
     // units to grow again: slot capacity exceeded / output buffer full
     i64 *retry_state;
     unsigned long long *n_retry_state;
-    i64 *retry_out;
+    i64 *retry_out;         // null: only counted
     unsigned long long *n_retry_out;
     u32 *error_flags;
 };
 
-// Bytes of one unit's state at `cap` node slots on graph G.
-size_t grow_state_bytes(const DevGraph &G, int cap);
+// Bytes of one unit's state at `cap` node slots on graph G (in shared memory or
+// in the arena, whose hash buckets are wider).
+size_t grow_state_bytes(const DevGraph &G, int cap, bool smem);
 // One unit per warp; `threads` = 32 * warps per CTA.
 int grow_launch(const GrowArgs &a, int blocks, int threads, size_t smem, cudaStream_t st);
 int grow_occupancy(const GrowArgs &a, int threads, size_t smem, int *blocks_per_sm);

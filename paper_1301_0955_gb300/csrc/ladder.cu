@@ -78,28 +78,27 @@ void pipe_free(GrowPipe &w) {
 
 int make_ladder(const DevGraph &G, i64 max_part_n, const mscd_params &p, std::vector<int> *ladder,
                 std::vector<bool> *in_smem) {
-    const size_t smem_budget = 220 * 1024;
     ladder->clear();
     int c0 = p.smem_slots;
-    if (c0 == 0) c0 = grow_state_bytes(G, 1024) * 4 <= smem_budget ? 1024 : 512;
-    if (grow_state_bytes(G, c0) > smem_budget) return MSCD_EINVAL;  // one unit's slots must fit a CTA
+    if (c0 == 0) c0 = grow_state_bytes(G, 1024, true) * 4 <= GROW_SMEM_MAX ? 1024 : 512;
+    if (grow_state_bytes(G, c0, true) > GROW_SMEM_MAX) return MSCD_EINVAL;  // one unit's slots must fit a CTA
     ladder->push_back(c0);
-    if (p.mid_slots > ladder->back() && grow_state_bytes(G, p.mid_slots) <= smem_budget)
+    if (p.mid_slots > ladder->back() && grow_state_bytes(G, p.mid_slots, true) <= GROW_SMEM_MAX)
         ladder->push_back(p.mid_slots);
     in_smem->assign(ladder->size(), true);
     // a community stays inside its seed's part: the part size bounds it
     i64 full = 32;
     while (full < max_part_n + 1) full <<= 1;
+    // global-memory classes; up to hash_smem_slots slots a class runs in shared
+    // memory too, where one unit's state fits it
     i64 cg = ladder->back();
-    if (p.global_slots > cg && cg < full) {
-        cg = std::min<i64>(p.global_slots, full);
-        ladder->push_back((int)cg);
-        in_smem->push_back(false);
-    }
+    bool first = true;
     while (cg < full) {
-        cg = std::min<i64>(cg * 8, full);
+        const i64 next = first && p.global_slots > cg ? p.global_slots : cg * 8;
+        first = false;
+        cg = std::min<i64>(next, full);
         ladder->push_back((int)cg);
-        in_smem->push_back(false);
+        in_smem->push_back(cg <= p.hash_smem_slots && grow_state_bytes(G, (int)cg, true) <= GROW_SMEM_MAX);
     }
     return MSCD_OK;
 }
@@ -118,8 +117,13 @@ int grow_units(GrowPipe &w, const GrowArgs &proto, i64 n_units, const std::vecto
         Task t = std::move(tasks.front());
         tasks.erase(tasks.begin());
         const int cap = ladder[t.cls];
-        const bool sm = in_smem[t.cls];
         const i64 n_work = t.all ? n_units : (i64)t.units.size();
+        // A few left-over units (at most one an SM) run in shared memory where a
+        // state of their class fits it: there is nothing to hide an arena's
+        // latency behind, and the launch lasts as long as its longest unit.
+        const bool sm = in_smem[t.cls] ||
+                        (!plain && t.cls > 0 && n_work <= w.sm_count && cap <= 32768 &&
+                         grow_state_bytes(G, cap, true) <= GROW_SMEM_MAX);
         // room for every list this launch can write (<= min(cap, n) each) when
         // that fits the budget; otherwise units that find it full are retried
         {
@@ -143,7 +147,7 @@ int grow_units(GrowPipe &w, const GrowArgs &proto, i64 n_units, const std::vecto
         a.retry_out = w.retry_b;
         a.n_retry_out = &w.ctr->n_retry_out;
         a.error_flags = &w.ctr->error_flags;
-        a.state_bytes = grow_state_bytes(G, cap);
+        a.state_bytes = grow_state_bytes(G, cap, sm);
         a.big_seed = t.cls == 0 ? proto.big_seed : nullptr;
         a.work_list = nullptr;
         i64 *list_dev = nullptr;
@@ -161,11 +165,14 @@ int grow_units(GrowPipe &w, const GrowArgs &proto, i64 n_units, const std::vecto
         int blocks = 0, threads = 32;
         size_t smem = 0;
         i64 chunk = n_work;  // work items per launch (the plain form's arena bounds it)
+        // few units go one to a CTA, two to a CTA, ... over all SMs: each is a chain
+        // of dependent steps, which neighbours only slow down
+        const int spread = (int)std::min<i64>(16, (n_work + w.sm_count - 1) / w.sm_count);
         if (sm) {
-            // as many one-warp units per CTA as fit 220 KiB (<= 16), one CTA per SM
+            // as many one-warp units per CTA as fit the shared memory (<= 16), one CTA per SM
             a.use_smem = 1;
-            a.bounds_smem = 0;
-            const int wpc = (int)std::max<size_t>(1, std::min<size_t>(16, (220 * 1024) / a.state_bytes));
+            int wpc = (int)std::max<size_t>(1, std::min<size_t>(16, GROW_SMEM_MAX / a.state_bytes));
+            if (!plain) wpc = std::max(1, std::min(wpc, spread));
             threads = 32 * wpc;
             smem = (size_t)wpc * a.state_bytes;
             int per_sm = 0;
@@ -175,26 +182,15 @@ int grow_units(GrowPipe &w, const GrowArgs &proto, i64 n_units, const std::vecto
             blocks = per_sm * w.sm_count;
         } else {
             a.use_smem = 0;
-            a.bounds_smem = 0;
-            a.hash_smem = 0;
             int wpc = GLOBAL_CTA_THREADS / 32;
             i64 per_sm_warps = w.p.global_warps_per_sm;
-            const size_t hash_bytes = 2 * (size_t)cap * (cap <= 32768 ? 2 : 4);
-            const size_t bounds_bytes = 8 * (size_t)(cap / 32);
-            if (cap <= w.p.hash_smem_slots) {
-                // hash table and bounds in shared memory, slot arrays in the arena:
-                // as many warps per CTA (one CTA per SM) as their tables fit
-                a.bounds_smem = 1;
-                a.hash_smem = 1;
-                a.smem_per_warp = (bounds_bytes + hash_bytes + 15) & ~(size_t)15;
-                wpc = (int)std::max<size_t>(1, std::min<size_t>(16, (220 * 1024) / a.smem_per_warp));
+            if (!plain) wpc = std::max(1, std::min(wpc, spread));
+            if (cap <= 32768) {
+                // group bounds (8 bytes per 32 slots and unit) in shared memory
+                a.smem_per_warp = 8 * (size_t)(cap / 32);
                 smem = (size_t)wpc * a.smem_per_warp;
-                per_sm_warps = wpc;
-            } else if (cap <= 16384) {
-                // group bounds (8 bytes per 32 slots and unit) in shared memory when small
-                a.bounds_smem = 1;
-                a.smem_per_warp = bounds_bytes;
-                smem = (size_t)wpc * a.smem_per_warp;
+            } else {
+                per_sm_warps = std::min<i64>(per_sm_warps, WIDE_MIN_BLOCKS * GLOBAL_CTA_THREADS / 32);
             }
             const size_t budget = (size_t)4 << 30;
             i64 warps = std::max<i64>(1, std::min<i64>((i64)(budget / a.state_bytes), (i64)w.sm_count * per_sm_warps));
