@@ -672,12 +672,11 @@ int run_impl(mscd_ctx *c, int32_t graph_id, const double *alphas, int32_t n_scal
         c->n_parts = P;
         c->nmi_succ.assign((size_t)P * S1, NAN);
         {
-            std::vector<double> pn(P);
-            for (int32_t s = 0; s + 1 < n_scales && rc == MSCD_OK; ++s) {
-                snprintf(stage, sizeof(stage), "stability between scales %d and %d", s, s + 1);
-                rc = nmi_between(c->scales[s], c->scales[s + 1], G.n, gr->part_off, P, pn.data(), st);
-                for (int32_t p = 0; p < P; ++p) c->nmi_succ[(size_t)p * S1 + s] = pn[p];
-            }
+            std::vector<double> pn((size_t)P * S1);
+            snprintf(stage, sizeof(stage), "stability");
+            rc = nmi_chain(c->scales.data(), n_scales, G.n, gr->part_off, P, pn.data(), st);
+            for (int32_t s = 0; s < S1; ++s)
+                for (int32_t p = 0; p < P; ++p) c->nmi_succ[(size_t)p * S1 + s] = pn[(size_t)s * P + p];
         }
         if (rc) break;
         c->win3.assign((size_t)P * n_scales, NAN);

@@ -855,8 +855,7 @@ int full_run(const DevGraph &G, i64 max_part_n, const double *alphas, int32_t n_
     if (rc) return rc;
     // stability between successive scales
     out->nmi.assign(std::max<size_t>(out->scales.size(), 1) - 1, NAN);
-    for (size_t s = 0; s + 1 < out->scales.size() && rc == MSCD_OK; ++s)
-        rc = nmi_between(out->scales[s], out->scales[s + 1], n, nullptr, 1, &out->nmi[s], st);
+    rc = nmi_chain(out->scales.data(), (int32_t)out->scales.size(), n, nullptr, 1, out->nmi.data(), st);
     if (rc) return rc;
     return out->status;
 }

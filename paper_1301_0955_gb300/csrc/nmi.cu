@@ -26,14 +26,21 @@
 //     largest active A community of the part; each A community walks its
 //     part's list in descending size and stops at the first B too small.
 // The intersections of the sharing pairs are counted by a warp per community:
-// it walks its members' lists of partner communities (the lanes spread over
-// one list at a time, whose entries are distinct) and counts in a
-// shared-memory hash; a community that meets too many partners is redone by
-// a whole CTA with a larger shared-memory table, and beyond that with a
-// global-memory table of its own.  Minima are kept as the bits of
-// non-negative doubles; the per-community terms are summed exactly (each
-// rounded once to a multiple of 2^-62, added in 128-bit integers), so the
-// value does not depend on the order of the additions.
+// it takes 32 of its members at a time, lays their lists of partner
+// communities end to end (the lanes then load 32 entries of several lists at
+// once, and the next ones while these are counted) and counts in a
+// shared-memory hash; a community with many members' lists to walk, or that
+// meets too many partners, is done by a whole CTA with a larger shared-memory
+// table, and beyond that with a global-memory table of its own.  A listed
+// partner of the last kind is disjoint iff it is not in the table.  Minima are
+// kept as the bits of non-negative doubles; the per-community terms are summed
+// exactly (each rounded once to a multiple of 2^-62, added in 128-bit
+// integers), so the value does not depend on the order of the additions.
+//
+// The terms h(c/n) come from a table over c (binary64 logarithms cost some
+// 2,700 cycles each here, and a candidate needs six).  All the pairs of a run
+// are queued without waiting; only where a scale has more communities than a
+// CTA's table holds does the host look at the counters of a pair.
 //
 // A graph that is a disjoint union of parts (independent graphs batched as
 // one) gets one NMI per part: a community lies inside one part (growth never
@@ -51,7 +58,10 @@ int ctx_device_of(mscd_ctx *c);
 namespace {
 
 constexpr int NMI_WARPS = 8;
-constexpr int NMI_TABLE = 512;  // shared-memory hash entries per warp (6 CTAs of 8 warps per SM)
+constexpr int NMI_TABLE = 512;  // shared-memory hash entries per warp (5 CTAs of 8 warps per SM)
+// Entries of partner lists a warp walks itself; more go to a CTA.  A warp takes
+// some 5 cycles an entry, so this bounds a launch's last warps to about 40 us.
+constexpr int WARP_ENTRIES = 16384;
 
 __device__ __forceinline__ double hterm(i64 c, double inv_n) {
     if (c <= 0) return 0.0;
@@ -59,18 +69,39 @@ __device__ __forceinline__ double hterm(i64 c, double inv_n) {
     return -p * log2(p);
 }
 
+// h(c/n) for the c of one part: from the table, or computed (no table: null).
+struct Terms {
+    const double *tab;
+    double inv_n;
+    __device__ __forceinline__ double operator()(i64 c) const { return tab ? tab[c] : hterm(c, inv_n); }
+};
+
+// tab[off[p] + p + c] = h(c / n_p), c = 0..n_p, for every part p.
+__global__ void fill_terms(const i64 *off, i32 P, i64 n, double *tab) {
+    for (i64 i = (i64)blockIdx.x * blockDim.x + threadIdx.x; i < n + P; i += (i64)gridDim.x * blockDim.x) {
+        i32 lo = 0, hi = P - 1;  // last part with off[p] + p <= i
+        while (off && lo < hi) {
+            const i32 mid = (lo + hi + 1) >> 1;
+            if (off[mid] + mid <= i) lo = mid;
+            else hi = mid - 1;
+        }
+        const i64 at = off ? off[lo] + lo : 0, np = off ? off[lo + 1] - off[lo] : n;
+        tab[i] = hterm(i - at, 1.0 / (double)np);
+    }
+}
+
 // Candidate H(A|B) for two communities of sizes sa, sb sharing n11 nodes, if
 // admitted; else +inf.
-__device__ __forceinline__ double cond_candidate(i64 n11, i64 sa, i64 sb, i64 n, double inv_n) {
+__device__ __forceinline__ double cond_candidate(i64 n11, i64 sa, i64 sb, i64 n, const Terms &H) {
     const i64 n10 = sa - n11, n01 = sb - n11, n00 = n - n11 - n10 - n01;
     const i64 lo1 = min(n11, n00), hi1 = max(n11, n00), lo2 = min(n01, n10), hi2 = max(n01, n10);
     if (lo1 == lo2 && hi1 == hi2) return __builtin_huge_val();
-    const double h11 = hterm(n11, inv_n), h00 = hterm(n00, inv_n), h01 = hterm(n01, inv_n), h10 = hterm(n10, inv_n);
+    const double h11 = H(n11), h00 = H(n00), h01 = H(n01), h10 = H(n10);
     if (!(h11 + h00 > h01 + h10)) return __builtin_huge_val();
-    return (h11 + h10 + h01 + h00) - (hterm(sb, inv_n) + hterm(n - sb, inv_n));
+    return (h11 + h10 + h01 + h00) - (H(sb) + H(n - sb));
 }
 
-__device__ __forceinline__ double entropy(i64 s, i64 n, double inv_n) { return hterm(s, inv_n) + hterm(n - s, inv_n); }
+__device__ __forceinline__ double entropy(i64 s, i64 n, const Terms &H) { return H(s) + H(n - s); }
 
 __device__ __forceinline__ unsigned long long min_bits(double v) {
     return (unsigned long long)__double_as_longlong(v > 0.0 ? v : 0.0);
@@ -146,13 +177,20 @@ __global__ void match_identical(const i64 *xptr, const i32 *xnodes, const u64 *x
 }
 
 // Part of every community (that of its first member; a community never spans
-// parts) and that part's node count.  No offsets: one part of n nodes.
-__global__ void comm_parts(const i64 *ptr, const i32 *nodes, i64 C, const i64 *off, i32 n_parts, i64 n, i32 *cp,
-                           i64 *cn) {
+// parts), that part's node count and its place in the table of terms.  No
+// offsets: one part of n nodes.
+struct CommParts {
+    i32 *cp = nullptr;
+    i64 *cn = nullptr;
+    i64 *ct = nullptr;
+};
+
+__global__ void comm_parts(const i64 *ptr, const i32 *nodes, i64 C, const i64 *off, i32 n_parts, i64 n, CommParts out) {
     for (i64 l = (i64)blockIdx.x * blockDim.x + threadIdx.x; l < C; l += (i64)gridDim.x * blockDim.x) {
         if (!off) {
-            cp[l] = 0;
-            cn[l] = n;
+            out.cp[l] = 0;
+            out.cn[l] = n;
+            out.ct[l] = 0;
             continue;
         }
         const i64 u = nodes[ptr[l]];
@@ -162,381 +200,478 @@ __global__ void comm_parts(const i64 *ptr, const i32 *nodes, i64 C, const i64 *o
             if (off[mid] <= u) lo = mid;
             else hi = mid - 1;
         }
-        cp[l] = lo;
-        cn[l] = off[lo + 1] - off[lo];
-    }
-}
-
-// Initial minima: 0 for communities with an identical partner, else H(C)
-// (the value when no partner is admitted); list the others.
-__global__ void init_best(const i64 *ptr, i64 C, const i64 *cn, const unsigned char *zero, unsigned long long *best,
-                          i32 *active, unsigned long long *n_active) {
-    for (i64 l = (i64)blockIdx.x * blockDim.x + threadIdx.x; l < C; l += (i64)gridDim.x * blockDim.x) {
-        if (zero[l]) {
-            best[l] = 0ull;
-        } else {
-            best[l] = min_bits(entropy(ptr[l + 1] - ptr[l], cn[l], 1.0 / (double)cn[l]));
-            active[atomicAdd(n_active, 1ull)] = (i32)l;
-        }
+        out.cp[l] = lo;
+        out.cn[l] = off[lo + 1] - off[lo];
+        out.ct[l] = off[lo] + lo;
     }
 }
 
 __device__ __forceinline__ u32 hash_comm(i32 l) { return (u32)l * 0x9E3779B1u; }
 
-struct DirArgs {
+// One direction of a pair of scales: H(A_k|B) for the communities of A
+// without an identical partner (the active ones).
+struct Direction {
     const i64 *aptr;
     const i32 *anodes;
-    const i32 *active;  // communities of A to process
-    i64 n_active;
+    i64 CA;
+    CommParts ap;
+    const unsigned char *zero;  // has an identical partner
+    i32 *active;
+    unsigned long long *n_active;
+    unsigned long long *best;   // per A community (bits of doubles)
+    unsigned long long *amax;   // per part: the largest active A community
     const i64 *bptr;
-    const i64 *mptr;    // node -> communities of B
+    i64 CB;
+    CommParts bp;
+    const i32 *mcnt;            // node -> number of communities of B,
+    const i64 *mptr;            // node -> communities of B
     const i32 *mlist;
-    const i64 *acn;            // per A community: node count of its part
-    unsigned long long *best;  // per A community (bits of doubles)
-    i64 *spill;                // positions in `active` redone with global tables
-    unsigned long long *n_spill;
+    // B communities that can meet an active A community of their part in an
+    // admitted disjoint pair, by part (boff), and the largest of each part
+    i32 *big;
+    i64 *boff;
+    unsigned long long *bmax, *bcount, *bfill;
+    i64 *spill, *spill2;        // positions in `active` left to the next tier
+    unsigned long long *n_spill, *n_spill2;
+};
+
+struct PairArgs {
+    Direction d[2];
+    i32 P;
+    const double *tab;
+    // work counters of the launches (zeroed before): communities are taken one
+    // at a time as warps or CTAs free up, since their costs differ by orders of
+    // magnitude; both directions share a launch
+    unsigned long long *next_warp, *next_block;
+    // global tables of the last tier
     const i64 *toff;
     i32 *tkey, *tcnt;
     i32 *tused;           // buckets each global table claimed, at the table's offset
     unsigned int *tfill;  // per community of a chunk: buckets claimed
-    // work counter of the launch (zeroed before it): communities are taken
-    // one at a time as warps or CTAs free up, since their costs differ by
-    // orders of magnitude
-    unsigned long long *next;
+    unsigned long long *next_global;
 };
 
-// Warp per active A community: intersections with every B community it meets
+// h(c/n) for the part of A's community k.
+__device__ __forceinline__ Terms terms_of(const PairArgs &a, const Direction &d, i32 k) {
+    return {a.tab ? a.tab + d.ap.ct[k] : nullptr, 1.0 / (double)d.ap.cn[k]};
+}
+
+// Initial minima: 0 for communities with an identical partner, else H(C)
+// (the value when no partner is admitted); list the others, and the largest
+// of them per part.  blockIdx.y: the direction (also below).
+__global__ void init_best(PairArgs a) {
+    const Direction &d = a.d[blockIdx.y];
+    for (i64 l = (i64)blockIdx.x * blockDim.x + threadIdx.x; l < d.CA; l += (i64)gridDim.x * blockDim.x) {
+        if (d.zero[l]) {
+            d.best[l] = 0ull;
+        } else {
+            const i64 s = d.aptr[l + 1] - d.aptr[l];
+            d.best[l] = min_bits(entropy(s, d.ap.cn[l], terms_of(a, d, (i32)l)));
+            d.active[atomicAdd(d.n_active, 1ull)] = (i32)l;
+            atomicMax(&d.amax[d.ap.cp[l]], (unsigned long long)s);
+        }
+    }
+}
+
+// B communities with 2(|B| + a) > n (n of B's part, a the largest active A
+// community of that part).  fill = 0 counts them per part, fill = 1 lists them.
+__global__ void list_big(PairArgs a, int fill) {
+    const Direction &d = a.d[blockIdx.y];
+    for (i64 l = (i64)blockIdx.x * blockDim.x + threadIdx.x; l < d.CB; l += (i64)gridDim.x * blockDim.x) {
+        const i32 p = d.bp.cp[l];
+        const i64 amax = (i64)d.amax[p], s = d.bptr[l + 1] - d.bptr[l];
+        if (amax == 0 || 2 * (s + amax) <= d.bp.cn[l]) continue;
+        if (fill) {
+            d.big[d.boff[p] + (i64)atomicAdd(&d.bfill[p], 1ull)] = (i32)l;
+        } else {
+            atomicAdd(&d.bcount[p], 1ull);
+            atomicMax(&d.bmax[p], (unsigned long long)s);
+        }
+    }
+}
+
+// Offsets of the parts' lists: a warp per direction.
+__global__ void big_offsets(PairArgs a) {
+    const Direction &d = a.d[blockIdx.y];
+    const int lane = threadIdx.x;
+    i64 at = 0;
+    for (i32 p0 = 0; p0 < a.P; p0 += 32) {
+        const i64 c = p0 + lane < a.P ? (i64)d.bcount[p0 + lane] : 0;
+        i64 x = c;
+        for (int o = 1; o < 32; o <<= 1) {
+            const i64 y = __shfl_up_sync(FULL_MASK, x, o);
+            if (lane >= o) x += y;
+        }
+        if (p0 + lane < a.P) d.boff[p0 + lane] = at + x - c;
+        at += __shfl_sync(FULL_MASK, x, 31);
+    }
+    if (lane == 0) d.boff[a.P] = at;
+}
+
+// f(l) for every community l of B that holds a member in anodes[e0, e1), at
+// most 32 members; once per member and community.  Warp-collective.
+template <class F>
+__device__ __forceinline__ void visit_partners(const Direction &d, i64 e0, i64 e1, F f) {
+    constexpr int AHEAD = 4;  // entries a lane has in flight
+    const int lane = threadIdx.x & 31;
+    i64 lo = 0;
+    int len = 0;
+    if (e0 + lane < e1) {
+        const i32 u = d.anodes[e0 + lane];
+        lo = d.mptr[u];
+        len = d.mcnt[u];
+    }
+    if (__any_sync(FULL_MASK, len > 1 << 25)) {  // the sums below would not fit
+        for (int i = 0; i < 32; ++i) {
+            const i64 b = __shfl_sync(FULL_MASK, lo, i);
+            const int m = __shfl_sync(FULL_MASK, len, i);
+            for (int t = lane; t < m; t += 32) f(d.mlist[b + t]);
+        }
+        return;
+    }
+    int incl = len;  // the lists end to end: member i's entries are incl - len .. incl
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(FULL_MASK, incl, o);
+        if (lane >= o) incl += y;
+    }
+    const int total = __shfl_sync(FULL_MASK, incl, 31);
+    const i64 first = lo - (incl - len);  // entry t of the whole is mlist[first + t]
+    for (int t0 = 0; t0 < total; t0 += 32 * AHEAD) {
+        i32 l[AHEAD];
+#pragma unroll
+        for (int j = 0; j < AHEAD; ++j) {
+            l[j] = -1;
+            if (t0 + 32 * j >= total) continue;
+            const int t = t0 + 32 * j + lane;
+            int i = 0;  // first member whose list ends beyond t
+#pragma unroll
+            for (int step = 16; step; step >>= 1)
+                if (__shfl_sync(FULL_MASK, incl, i + step - 1) <= t) i += step;
+            const i64 b = __shfl_sync(FULL_MASK, first, i);
+            if (t < total) l[j] = d.mlist[b + t];
+        }
+#pragma unroll
+        for (int j = 0; j < AHEAD; ++j)
+            if (l[j] >= 0) f(l[j]);
+    }
+}
+
+// A hash of partner communities and how many nodes they share with A's.
+struct Counts {
+    i32 *keys, *cnts;
+    u32 mask;
+    // Count one node shared with l; true: l is new, in the bucket `at`.
+    __device__ __forceinline__ bool add(i32 l, u32 &at) const {
+        u32 h = hash_comm(l) & mask;
+        bool fresh = false;
+        for (u32 p = 0; p <= mask; ++p) {
+            i32 cur = keys[h];
+            if (cur == -1) {
+                cur = atomicCAS(&keys[h], -1, l);
+                if (cur == -1) {
+                    fresh = true;
+                    cur = l;
+                }
+            }
+            if (cur == l) {
+                atomicAdd(&cnts[h], 1);
+                break;
+            }
+            h = (h + 1u) & mask;
+        }
+        at = h;
+        return fresh;
+    }
+    __device__ __forceinline__ bool has(i32 l) const {
+        u32 h = hash_comm(l) & mask;
+        for (u32 p = 0; p <= mask; ++p) {
+            const i32 cur = keys[h];
+            if (cur == l) return true;
+            if (cur == -1) return false;
+            h = (h + 1u) & mask;
+        }
+        return false;
+    }
+};
+
+// The least candidate of community k (size sa): this thread's share of its
+// partners, bucket(t) for t < nf, and of the listed ones it shares nothing
+// with (|A| + |B| > n/2).  `rank` of `size` threads.
+template <class B>
+__device__ __forceinline__ double least_candidate(const PairArgs &a, const Direction &d, i32 k, const Counts &C, int nf,
+                                                  B bucket, int rank, int size) {
+    const i64 sa = d.aptr[k + 1] - d.aptr[k], n = d.ap.cn[k];
+    const Terms H = terms_of(a, d, k);
+    double bx = __builtin_huge_val();
+    for (int t = rank; t < nf; t += size) {
+        const u32 h = bucket(t);
+        const i32 l = C.keys[h];
+        bx = min(bx, cond_candidate(C.cnts[h], sa, d.bptr[l + 1] - d.bptr[l], n, H));
+    }
+    const i32 p = d.ap.cp[k];
+    if (2 * (sa + (i64)d.bmax[p]) > n)
+        for (i64 j = d.boff[p] + rank; j < d.boff[p + 1]; j += size) {
+            const i32 l = d.big[j];
+            const i64 sb = d.bptr[l + 1] - d.bptr[l];
+            if (2 * (sa + sb) > n && !C.has(l)) bx = min(bx, cond_candidate(0, sa, sb, n, H));
+        }
+    return bx;
+}
+
+__device__ __forceinline__ double warp_min(double x) {
+    for (int o = 16; o; o >>= 1) x = min(x, __shfl_xor_sync(FULL_MASK, x, o));
+    return x;
+}
+
+// Warp per active community: intersections with every B community it meets
 // (shared-memory hash), minimum admitted candidate.
 // The buckets a community fills are listed as they are claimed, so the scan
 // and the reset after it touch only those (the table is cleared once).
-__global__ void __launch_bounds__(NMI_WARPS * 32) pairs_smem(DirArgs a) {
+__global__ void __launch_bounds__(NMI_WARPS * 32) pairs_warp(const __grid_constant__ PairArgs a) {
     __shared__ i32 skey[NMI_WARPS][NMI_TABLE];
     __shared__ i32 scnt[NMI_WARPS][NMI_TABLE];
     __shared__ unsigned short sused[NMI_WARPS][NMI_TABLE / 2];
     __shared__ int sfill[NMI_WARPS];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    i32 *keys = skey[w];
-    i32 *cnts = scnt[w];
+    const Counts C = {skey[w], scnt[w], NMI_TABLE - 1};
     unsigned short *used = sused[w];
     for (int t = lane; t < NMI_TABLE; t += 32) {
-        keys[t] = -1;
-        cnts[t] = 0;
+        C.keys[t] = -1;
+        C.cnts[t] = 0;
     }
     __syncwarp();
+    const i64 n0 = (i64)*a.d[0].n_active, n1 = (i64)*a.d[1].n_active;
     for (;;) {
         unsigned long long qq = 0;
-        if (lane == 0) qq = atomicAdd(a.next, 1ull);
-        const i64 q = (i64)__shfl_sync(FULL_MASK, qq, 0);
-        if (q >= a.n_active) break;
-        const i32 k = a.active[q];
-        if (lane == 0) sfill[w] = 0;
-        __syncwarp();
-        bool over = false;
-        for (i64 e = a.aptr[k]; e < a.aptr[k + 1] && !over; ++e) {
-            const i32 u = a.anodes[e];
-            for (i64 j = a.mptr[u] + lane; j < a.mptr[u + 1]; j += 32) {
-                const i32 l = a.mlist[j];
-                u32 h = hash_comm(l) & (NMI_TABLE - 1);
-                for (int p = 0; p < NMI_TABLE; ++p) {
-                    i32 cur = keys[h];
-                    if (cur == -1) {
-                        cur = atomicCAS(&keys[h], -1, l);
-                        if (cur == -1) {
-                            const int f = atomicAdd(&sfill[w], 1);
-                            if (f >= NMI_TABLE / 2) over = true;
-                            else used[f] = (unsigned short)h;
-                            cur = l;
-                        }
+        if (lane == 0) qq = atomicAdd(a.next_warp, 1ull);
+        i64 q = (i64)__shfl_sync(FULL_MASK, qq, 0);
+        if (q >= n0 + n1) break;
+        const Direction &d = a.d[q >= n0 ? 1 : 0];
+        if (q >= n0) q -= n0;
+        const i32 k = d.active[q];
+        const i64 e0 = d.aptr[k], e1 = d.aptr[k + 1];
+        i64 entries = 0;
+#pragma unroll 4
+        for (i64 e = e0 + lane; e < e1; e += 32) entries += d.mcnt[d.anodes[e]];
+        for (int o = 16; o; o >>= 1) entries += __shfl_xor_sync(FULL_MASK, entries, o);
+        bool over = entries > WARP_ENTRIES;
+        if (!over) {
+            if (lane == 0) sfill[w] = 0;
+            __syncwarp();
+            for (i64 e = e0; e < e1 && !over; e += 32) {
+                visit_partners(d, e, min(e + 32, e1), [&](i32 l) {
+                    u32 h;
+                    if (C.add(l, h)) {
+                        const int f = atomicAdd(&sfill[w], 1);
+                        if (f >= NMI_TABLE / 2) over = true;
+                        else used[f] = (unsigned short)h;
                     }
-                    if (cur == l) {
-                        atomicAdd(&cnts[h], 1);
-                        break;
-                    }
-                    h = (h + 1u) & (NMI_TABLE - 1);
-                }
-            }
-            over = __any_sync(FULL_MASK, over);
-        }
-        __syncwarp();
-        if (over) {
-            if (lane == 0) a.spill[atomicAdd(a.n_spill, 1ull)] = q;
-            for (int t = lane; t < NMI_TABLE; t += 32) {  // more buckets than listed: clear all
-                keys[t] = -1;
-                cnts[t] = 0;
+                });
+                over = __any_sync(FULL_MASK, over);
             }
             __syncwarp();
+            if (over) {  // more buckets than listed: clear all
+                for (int t = lane; t < NMI_TABLE; t += 32) {
+                    C.keys[t] = -1;
+                    C.cnts[t] = 0;
+                }
+                __syncwarp();
+            }
+        }
+        if (over) {
+            if (lane == 0) d.spill[atomicAdd(d.n_spill, 1ull)] = q;
             continue;
         }
         const int nf = sfill[w];
-        const i64 sa = a.aptr[k + 1] - a.aptr[k], n = a.acn[k];
-        const double inv_n = 1.0 / (double)n;
-        double bx = __longlong_as_double((long long)a.best[k]);
-        for (int t = lane; t < nf; t += 32) {
-            const int h = used[t];
-            const i32 l = keys[h];
-            bx = min(bx, cond_candidate(cnts[h], sa, a.bptr[l + 1] - a.bptr[l], n, inv_n));
-            keys[h] = -1;
-            cnts[h] = 0;
-        }
-        for (int o = 16; o; o >>= 1) bx = min(bx, __shfl_xor_sync(FULL_MASK, bx, o));
-        if (lane == 0) a.best[k] = min_bits(bx);
+        const double bx =
+            warp_min(least_candidate(a, d, k, C, nf, [&](int t) { return (u32)used[t]; }, lane, 32));
         __syncwarp();
-    }
-}
-
-// CTA per listed community (positions in `active`): the same with a global
-// table of its own, the community's members spread over the CTA's warps (these
-// communities meet thousands of partners through millions of incidences).
-constexpr int GLB_WARPS = 16;
-
-__global__ void __launch_bounds__(GLB_WARPS * 32) pairs_global(DirArgs a, const i64 *list, i64 nk) {
-    __shared__ double wmin[GLB_WARPS];
-    __shared__ i64 rnext;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (;;) {
-        if (threadIdx.x == 0) rnext = (i64)atomicAdd(a.next, 1ull);
-        __syncthreads();
-        const i64 r = rnext;
-        if (r >= nk) break;
-        const i32 k = a.active[list[r]];
-        i32 *keys = a.tkey + a.toff[r];
-        i32 *cnts = a.tcnt + a.toff[r];
-        i32 *used = a.tused + a.toff[r];
-        unsigned int *fill = a.tfill + r;
-        const u32 tm = (u32)(a.toff[r + 1] - a.toff[r] - 1);
-        for (i64 e = a.aptr[k] + w; e < a.aptr[k + 1]; e += GLB_WARPS) {
-            const i32 u = a.anodes[e];
-            for (i64 j = a.mptr[u] + lane; j < a.mptr[u + 1]; j += 32) {
-                const i32 l = a.mlist[j];
-                u32 h = hash_comm(l) & tm;
-                for (u32 p = 0; p <= tm; ++p) {
-                    i32 cur = keys[h];
-                    if (cur == -1) {
-                        cur = atomicCAS(&keys[h], -1, l);
-                        if (cur == -1) {
-                            used[atomicAdd(fill, 1u)] = (i32)h;
-                            cur = l;
-                        }
-                    }
-                    if (cur == l) {
-                        atomicAdd(&cnts[h], 1);
-                        break;
-                    }
-                    h = (h + 1u) & tm;
-                }
-            }
+        for (int t = lane; t < nf; t += 32) {
+            C.keys[used[t]] = -1;
+            C.cnts[used[t]] = 0;
         }
-        __syncthreads();
-        const i64 sa = a.aptr[k + 1] - a.aptr[k], n = a.acn[k];
-        const double inv_n = 1.0 / (double)n;
-        double bx = __builtin_huge_val();
-        // only the claimed buckets, emptied again for the table's next user
-        const u32 nf = *(volatile unsigned int *)fill;
-        for (u32 t = threadIdx.x; t < nf; t += GLB_WARPS * 32) {
-            const i32 hh = used[t];
-            const i32 l = keys[hh];
-            bx = min(bx, cond_candidate(cnts[hh], sa, a.bptr[l + 1] - a.bptr[l], n, inv_n));
-            keys[hh] = -1;
-            cnts[hh] = 0;
-        }
-        for (int o = 16; o; o >>= 1) bx = min(bx, __shfl_xor_sync(FULL_MASK, bx, o));
-        if (lane == 0) wmin[w] = bx;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double m = __longlong_as_double((long long)a.best[k]);
-            for (int q = 0; q < GLB_WARPS; ++q) m = min(m, wmin[q]);
-            a.best[k] = min_bits(m);
-        }
-        __syncthreads();
+        if (lane == 0) d.best[k] = min_bits(min(bx, __longlong_as_double((long long)d.best[k])));
+        __syncwarp();
     }
 }
 
 constexpr int BLK_WARPS = 16;
 constexpr int BLK_TABLE = 8192;  // shared-memory hash entries of one CTA (72 KB: 3 CTAs per SM)
 
-// CTA per community spilled by pairs_smem: its members are spread over the
+// Members a warp of a CTA takes at a time: all of the CTA's warps get some.
+__device__ __forceinline__ i64 member_chunk(i64 members, int warps) {
+    return min((members + warps - 1) / warps, (i64)32);
+}
+
+// CTA per community left by pairs_warp: its members are spread over the
 // warps, an 8192-entry shared-memory table counts the intersections; a
 // community meeting more than half of that is listed for pairs_global.
-__global__ void __launch_bounds__(BLK_WARPS * 32) pairs_block(DirArgs a, const i64 *list, i64 nk, i64 *spill2,
-                                                              unsigned long long *n_spill2) {
+__global__ void __launch_bounds__(BLK_WARPS * 32) pairs_block(const __grid_constant__ PairArgs a) {
     extern __shared__ i32 tab[];
-    i32 *keys = tab, *cnts = tab + BLK_TABLE;
+    const Counts C = {tab, tab + BLK_TABLE, BLK_TABLE - 1};
     unsigned short *used = (unsigned short *)(tab + 2 * BLK_TABLE);  // [BLK_TABLE / 2]
     __shared__ int fill, over;
     __shared__ double wmin[BLK_WARPS];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     __shared__ i64 rnext;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const i64 n0 = (i64)*a.d[0].n_spill, n1 = (i64)*a.d[1].n_spill;
+    if (n0 + n1 == 0) return;
     for (int t = threadIdx.x; t < BLK_TABLE; t += BLK_WARPS * 32) {
-        keys[t] = -1;
-        cnts[t] = 0;
+        C.keys[t] = -1;
+        C.cnts[t] = 0;
     }
     for (;;) {
-        if (threadIdx.x == 0) rnext = (i64)atomicAdd(a.next, 1ull);
         __syncthreads();
-        const i64 r = rnext;
-        if (r >= nk) break;
-        const i64 q = list[r];
-        const i32 k = a.active[q];
         if (threadIdx.x == 0) {
+            rnext = (i64)atomicAdd(a.next_block, 1ull);
             fill = 0;
             over = 0;
         }
         __syncthreads();
-        for (i64 e = a.aptr[k] + w; e < a.aptr[k + 1]; e += BLK_WARPS) {
+        i64 r = rnext;
+        if (r >= n0 + n1) break;
+        const Direction &d = a.d[r >= n0 ? 1 : 0];
+        if (r >= n0) r -= n0;
+        const i64 q = d.spill[r];
+        const i32 k = d.active[q];
+        const i64 e0 = d.aptr[k], e1 = d.aptr[k + 1], step = member_chunk(e1 - e0, BLK_WARPS);
+        for (i64 e = e0 + w * step; e < e1; e += BLK_WARPS * step) {
             if (*(volatile int *)&over) break;
-            const i32 u = a.anodes[e];
-            for (i64 j = a.mptr[u] + lane; j < a.mptr[u + 1]; j += 32) {
-                const i32 l = a.mlist[j];
-                u32 h = hash_comm(l) & (BLK_TABLE - 1);
-                for (int p = 0; p < BLK_TABLE; ++p) {
-                    i32 cur = keys[h];
-                    if (cur == -1) {
-                        cur = atomicCAS(&keys[h], -1, l);
-                        if (cur == -1) {
-                            const int f = atomicAdd(&fill, 1);
-                            if (f >= BLK_TABLE / 2) over = 1;
-                            else used[f] = (unsigned short)h;
-                            cur = l;
-                        }
-                    }
-                    if (cur == l) {
-                        atomicAdd(&cnts[h], 1);
-                        break;
-                    }
-                    h = (h + 1u) & (BLK_TABLE - 1);
+            visit_partners(d, e, min(e + step, e1), [&](i32 l) {
+                u32 h;
+                if (C.add(l, h)) {
+                    const int f = atomicAdd(&fill, 1);
+                    if (f >= BLK_TABLE / 2) over = 1;
+                    else used[f] = (unsigned short)h;
                 }
-            }
+            });
         }
         __syncthreads();
         if (over) {
-            if (threadIdx.x == 0) spill2[atomicAdd(n_spill2, 1ull)] = q;
+            if (threadIdx.x == 0) d.spill2[atomicAdd(d.n_spill2, 1ull)] = q;
             for (int t = threadIdx.x; t < BLK_TABLE; t += BLK_WARPS * 32) {  // clear all
-                keys[t] = -1;
-                cnts[t] = 0;
+                C.keys[t] = -1;
+                C.cnts[t] = 0;
             }
-            __syncthreads();
             continue;
         }
         const int nf = fill;
-        const i64 sa = a.aptr[k + 1] - a.aptr[k], n = a.acn[k];
-        const double inv_n = 1.0 / (double)n;
-        double bx = __builtin_huge_val();
-        for (int t = threadIdx.x; t < nf; t += BLK_WARPS * 32) {
-            const int h = used[t];
-            const i32 l = keys[h];
-            bx = min(bx, cond_candidate(cnts[h], sa, a.bptr[l + 1] - a.bptr[l], n, inv_n));
-            keys[h] = -1;
-            cnts[h] = 0;
-        }
-        for (int o = 16; o; o >>= 1) bx = min(bx, __shfl_xor_sync(FULL_MASK, bx, o));
+        const double bx = warp_min(least_candidate(a, d, k, C, nf, [&](int t) { return (u32)used[t]; },
+                                                   (int)threadIdx.x, BLK_WARPS * 32));
         if (lane == 0) wmin[w] = bx;
         __syncthreads();
+        for (int t = threadIdx.x; t < nf; t += BLK_WARPS * 32) {
+            C.keys[used[t]] = -1;
+            C.cnts[used[t]] = 0;
+        }
         if (threadIdx.x == 0) {
-            double m = __longlong_as_double((long long)a.best[k]);
+            double m = __longlong_as_double((long long)d.best[k]);
             for (int i = 0; i < BLK_WARPS; ++i) m = min(m, wmin[i]);
-            a.best[k] = min_bits(m);
+            d.best[k] = min_bits(m);
+        }
+    }
+}
+
+// CTA per listed community (positions in `active`): the same with a global
+// table of its own (these communities meet thousands of partners through
+// millions of incidences).
+constexpr int GLB_WARPS = 16;
+
+__global__ void __launch_bounds__(GLB_WARPS * 32) pairs_global(const __grid_constant__ PairArgs a, int dir,
+                                                               const i64 *list, i64 nk) {
+    __shared__ double wmin[GLB_WARPS];
+    __shared__ i64 rnext;
+    const Direction &d = a.d[dir];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (;;) {
+        if (threadIdx.x == 0) rnext = (i64)atomicAdd(a.next_global, 1ull);
+        __syncthreads();
+        const i64 r = rnext;
+        if (r >= nk) break;
+        const i32 k = d.active[list[r]];
+        const Counts C = {a.tkey + a.toff[r], a.tcnt + a.toff[r], (u32)(a.toff[r + 1] - a.toff[r] - 1)};
+        i32 *used = a.tused + a.toff[r];
+        unsigned int *fill = a.tfill + r;
+        const i64 e0 = d.aptr[k], e1 = d.aptr[k + 1], step = member_chunk(e1 - e0, GLB_WARPS);
+        for (i64 e = e0 + w * step; e < e1; e += GLB_WARPS * step)
+            visit_partners(d, e, min(e + step, e1), [&](i32 l) {
+                u32 h;
+                if (C.add(l, h)) used[atomicAdd(fill, 1u)] = (i32)h;
+            });
+        __syncthreads();
+        // only the claimed buckets, emptied again for the table's next user
+        const u32 nf = *(volatile unsigned int *)fill;
+        const double bx = warp_min(least_candidate(a, d, k, C, (int)nf, [&](int t) { return (u32)used[t]; },
+                                                   (int)threadIdx.x, GLB_WARPS * 32));
+        if (lane == 0) wmin[w] = bx;
+        __syncthreads();
+        for (u32 t = threadIdx.x; t < nf; t += GLB_WARPS * 32) {
+            C.keys[used[t]] = -1;
+            C.cnts[used[t]] = 0;
+        }
+        if (threadIdx.x == 0) {
+            double m = __longlong_as_double((long long)d.best[k]);
+            for (int q = 0; q < GLB_WARPS; ++q) m = min(m, wmin[q]);
+            d.best[k] = min_bits(m);
         }
         __syncthreads();
     }
 }
 
-// Table size of each spilled community: 2 * min(incidences, |B|) rounded up
-// to a power of two.
-__global__ void spill_sizes(const i64 *list, i64 nk, const i32 *active, const i64 *aptr, const i32 *anodes,
-                            const i32 *bcnt, i64 CB, i64 *tsz) {
+// Table size of each community of the last tier: 2 * min(incidences, |B|)
+// rounded up to a power of two.
+__global__ void spill_sizes(const i64 *list, i64 nk, Direction d, i64 *tsz) {
     const int lane = threadIdx.x & 31;
     const i64 warps = (i64)gridDim.x * (blockDim.x >> 5);
     for (i64 r = (i64)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < nk; r += warps) {
-        const i32 k = active[list[r]];
+        const i32 k = d.active[list[r]];
         i64 s = 0;
-        for (i64 e = aptr[k] + lane; e < aptr[k + 1]; e += 32) s += bcnt[anodes[e]];
+        for (i64 e = d.aptr[k] + lane; e < d.aptr[k + 1]; e += 32) s += d.mcnt[d.anodes[e]];
         for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(FULL_MASK, s, o);
-        s = min(s, CB);
+        s = min(s, d.CB);
         i64 t = 2;
         while (t < 2 * s) t <<= 1;
         if (lane == 0) tsz[r] = t;
     }
 }
 
-// Disjoint pairs that can be admitted (|A| + |B| > n/2).
-// The candidate B communities grouped by part (boff: offsets per part) and
-// in descending size inside a part, so that an A community meets only those
-// of its own part and stops at the first one with 2(|A| + |B|) <= n: warp
-// per active A, lanes over its part's list.
-__global__ void disjoint_pairs(const i64 *aptr, const i32 *anodes, const i32 *active, i64 n_active,
-                               const i64 *bptr, const i32 *bnodes, const i32 *big, const i64 *boff,
-                               const i32 *acp, const i64 *acn, unsigned long long *best) {
-    const int lane = threadIdx.x & 31;
-    const i64 warps = (i64)gridDim.x * (blockDim.x >> 5);
-    for (i64 q = (i64)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); q < n_active; q += warps) {
-        const i32 k = active[q];
-        const i32 p = acp[k];
-        const i64 sa = aptr[k + 1] - aptr[k], n = acn[k];
-        double bx = __builtin_huge_val();
-        for (i64 j = boff[p] + lane; j < boff[p + 1]; j += 32) {
-            const i32 l = big[j];
-            const i64 sb = bptr[l + 1] - bptr[l];
-            if (2 * (sa + sb) <= n) break;  // every later entry of this lane is smaller
-            const i32 *x = anodes + aptr[k], *y = bnodes + bptr[l];
-            i64 i = 0, jj = 0;
-            bool meet = false;
-            while (i < sa && jj < sb) {
-                if (x[i] < y[jj]) ++i;
-                else if (x[i] > y[jj]) ++jj;
-                else {
-                    meet = true;
-                    break;
-                }
-            }
-            if (!meet) bx = min(bx, cond_candidate(0, sa, sb, n, 1.0 / (double)n));
-        }
-        for (int o = 16; o; o >>= 1) bx = min(bx, __shfl_xor_sync(FULL_MASK, bx, o));
-        if (lane == 0 && bx < __builtin_huge_val()) atomicMin(&best[k], min_bits(bx));
-    }
-}
-
-__global__ void gather_parts(const i32 *big, i64 nbig, const i32 *cp, const i64 *ptr, i32 *out, i64 *size) {
-    for (i64 i = (i64)blockIdx.x * blockDim.x + threadIdx.x; i < nbig; i += (i64)gridDim.x * blockDim.x) {
-        out[i] = cp[big[i]];
-        size[i] = ptr[big[i] + 1] - ptr[big[i]];
-    }
-}
-
-// Largest active A community of every part.
-__global__ void active_max_size(const i64 *aptr, const i32 *active, i64 n_active, const i32 *acp,
-                                unsigned long long *amax) {
-    for (i64 q = (i64)blockIdx.x * blockDim.x + threadIdx.x; q < n_active; q += (i64)gridDim.x * blockDim.x) {
-        const i32 k = active[q];
-        atomicMax(&amax[acp[k]], (unsigned long long)(aptr[k + 1] - aptr[k]));
-    }
-}
-
-// B communities with 2(|B| + a) > n (n of B's part, a the largest active A
-// community of that part): the only ones that can meet an active A community
-// of their part in an admitted disjoint pair.
-__global__ void list_big(const i64 *ptr, i64 C, const i32 *cp, const i64 *cn, const unsigned long long *amax,
-                         i32 *big, unsigned long long *nbig) {
-    for (i64 l = (i64)blockIdx.x * blockDim.x + threadIdx.x; l < C; l += (i64)gridDim.x * blockDim.x) {
-        const i64 a = (i64)amax[cp[l]];
-        if (a > 0 && 2 * (ptr[l + 1] - ptr[l] + a) > cn[l]) big[atomicAdd(nbig, 1ull)] = (i32)l;
-    }
-}
-
 // Normalised term H(A_k|B) / H(A_k) in [0, 1] (the minimum never exceeds its
 // initial value H(A_k), computed the same way), added to its part's total as
-// an integer multiple of 2^-62 in 128 bits: acc[2p] low word, acc[2p+1] carries.
-__global__ void normalise_sum(const i64 *ptr, i64 C, const i64 *cn, const i32 *cp,
-                              const unsigned long long *best, unsigned long long *acc,
-                              unsigned long long *count) {
-    for (i64 k = (i64)blockIdx.x * blockDim.x + threadIdx.x; k < C; k += (i64)gridDim.x * blockDim.x) {
-        const i64 n = cn[k];
-        const double H = entropy(ptr[k + 1] - ptr[k], n, 1.0 / (double)n);
-        const double t = H > 0.0 ? __longlong_as_double((long long)best[k]) / H : 0.0;
-        const unsigned long long q = (unsigned long long)__double2ll_rn(fmin(fmax(t, 0.0), 1.0) * 0x1p62);
-        const i32 p = cp[k];
-        const unsigned long long old = atomicAdd(&acc[2 * p], q);
-        if (old + q < old) atomicAdd(&acc[2 * p + 1], 1ull);
-        atomicAdd(&count[p], 1ull);
+// an integer multiple of 2^-62 in 128 bits.  acc: per part, the two
+// directions' sums (low word, carries), then their counts.  One part: the
+// warps' sums are added first (every community on one address otherwise).
+__global__ void normalise_sum(PairArgs a, unsigned long long *acc) {
+    const Direction &d = a.d[blockIdx.y];
+    unsigned long long *sum = acc + (size_t)blockIdx.y * 2 * a.P, *count = acc + (size_t)(4 + blockIdx.y) * a.P;
+    const i64 stride = (i64)gridDim.x * blockDim.x;
+    for (i64 k0 = (i64)blockIdx.x * blockDim.x; k0 < d.CA; k0 += stride) {
+        const i64 k = k0 + threadIdx.x;
+        unsigned long long q = 0;
+        if (k < d.CA) {
+            const double H = entropy(d.aptr[k + 1] - d.aptr[k], d.ap.cn[k], terms_of(a, d, (i32)k));
+            const double t = H > 0.0 ? __longlong_as_double((long long)d.best[k]) / H : 0.0;
+            q = (unsigned long long)__double2ll_rn(fmin(fmax(t, 0.0), 1.0) * 0x1p62);
+        }
+        if (a.P == 1) {
+            unsigned long long lo = q, hi = 0;
+            for (int o = 16; o; o >>= 1) {
+                const unsigned long long l2 = __shfl_xor_sync(FULL_MASK, lo, o), h2 = __shfl_xor_sync(FULL_MASK, hi, o);
+                lo += l2;
+                hi += h2 + (lo < l2 ? 1ull : 0ull);
+            }
+            const int live = __popc(__ballot_sync(FULL_MASK, k < d.CA));
+            if ((threadIdx.x & 31) == 0 && live) {
+                const unsigned long long old = atomicAdd(&sum[0], lo);
+                hi += old + lo < old ? 1ull : 0ull;
+                if (hi) atomicAdd(&sum[1], hi);
+                atomicAdd(&count[0], (unsigned long long)live);
+            }
+        } else if (k < d.CA) {
+            const i32 p = d.ap.cp[k];
+            const unsigned long long old = atomicAdd(&sum[2 * p], q);
+            if (old + q < old) atomicAdd(&sum[2 * p + 1], 1ull);
+            atomicAdd(&count[p], 1ull);
+        }
     }
 }
 
@@ -546,6 +681,10 @@ int dev_alloc(T **p, i64 count, cudaStream_t st) {
 }
 
 const unsigned GB = 152 * 16;
+constexpr i64 TERMS_MAX = (i64)1 << 26;  // nodes up to which the terms are tabled (8 bytes each)
+
+// CTAs of 256 threads for m threads of work.
+unsigned grid_of(i64 m) { return (unsigned)std::max<i64>(1, std::min<i64>((m + 255) / 256, GB)); }
 
 // node -> communities map of B.
 struct Memberships {
@@ -558,292 +697,259 @@ int build_memberships(const ScaleResult &B, i64 n, Memberships *M, cudaStream_t 
     i64 *tmp = nullptr;
     int rc = MSCD_OK;
     do {
-        if ((rc = dev_alloc(&M->cnt, n, st))) break;
+        if ((rc = dev_alloc(&M->cnt, 2 * n, st))) break;
+        cursor = M->cnt + n;
         if ((rc = dev_alloc(&M->ptr, n + 1, st))) break;
         if ((rc = dev_alloc(&M->list, B.n_nodes, st))) break;
-        if ((rc = dev_alloc(&cursor, n, st))) break;
         if ((rc = dev_alloc(&tmp, n + 1, st))) break;
-        if ((rc = cuda_status(cudaMemsetAsync(M->cnt, 0, n * sizeof(i32), st)))) break;
-        if ((rc = cuda_status(cudaMemsetAsync(cursor, 0, n * sizeof(i32), st)))) break;
-        count_memberships<<<GB, 256, 0, st>>>(B.comm_nodes, B.n_nodes, M->cnt); note_launch();
-        widen_i32<<<GB, 256, 0, st>>>(M->cnt, n, tmp); note_launch();
+        if ((rc = cuda_status(cudaMemsetAsync(M->cnt, 0, 2 * n * sizeof(i32), st)))) break;
+        count_memberships<<<grid_of(B.n_nodes), 256, 0, st>>>(B.comm_nodes, B.n_nodes, M->cnt); note_launch();
+        widen_i32<<<grid_of(n), 256, 0, st>>>(M->cnt, n, tmp); note_launch();
         if ((rc = scan_exclusive_i64(tmp, M->ptr, n, M->ptr + n, st))) break;
-        fill_memberships<<<GB, 256, 0, st>>>(B.comm_ptr, B.comm_nodes, B.n_comms, M->ptr, cursor, M->list); note_launch();
+        fill_memberships<<<grid_of(32 * B.n_comms), 256, 0, st>>>(B.comm_ptr, B.comm_nodes, B.n_comms, M->ptr, cursor,
+                                                                  M->list); note_launch();
     } while (0);
-    cudaFreeAsync(cursor, st);
     cudaFreeAsync(tmp, st);
     return rc;
 }
 
-void free_memberships(Memberships *M, cudaStream_t st) {
-    cudaFreeAsync(M->cnt, st);
-    cudaFreeAsync(M->ptr, st);
-    cudaFreeAsync(M->list, st);
-}
-
-// Minimum admitted H(A_k|B) for every active A_k into best[] (one direction).
-// Per-community part data of one scale's communities.
-struct CommParts {
-    i32 *cp = nullptr;  // part index
-    i64 *cn = nullptr;  // node count of that part
+// What the pairs of a scale with its neighbours share.
+struct ScaleData {
+    CommParts parts;
+    Memberships members;
 };
 
-int one_direction(const ScaleResult &A, const ScaleResult &B, const Memberships &MB, const CommParts &PA,
-                  const CommParts &PB, int32_t P, const i32 *active, i64 n_active, unsigned long long *best,
-                  cudaStream_t st) {
-    i64 *spill = nullptr, *spill2 = nullptr, *tsz = nullptr, *toff = nullptr, *dboff = nullptr, *bsize = nullptr;
-    i32 *bpart = nullptr;
-    i32 *tkey = nullptr, *tcnt = nullptr, *tused = nullptr, *big = nullptr;
+void free_scale(ScaleData *s, cudaStream_t st) {
+    cudaFreeAsync(s->parts.cp, st);
+    cudaFreeAsync(s->parts.cn, st);
+    cudaFreeAsync(s->parts.ct, st);
+    cudaFreeAsync(s->members.cnt, st);
+    cudaFreeAsync(s->members.ptr, st);
+    cudaFreeAsync(s->members.list, st);
+    *s = ScaleData{};
+}
+
+int build_scale(const ScaleResult &R, i64 n, const i64 *part_off, int32_t P, ScaleData *s, cudaStream_t st) {
+    int rc = dev_alloc(&s->parts.cp, R.n_comms, st);
+    if (!rc) rc = dev_alloc(&s->parts.cn, R.n_comms, st);
+    if (!rc) rc = dev_alloc(&s->parts.ct, R.n_comms, st);
+    if (rc) return rc;
+    comm_parts<<<grid_of(R.n_comms), 256, 0, st>>>(R.comm_ptr, R.comm_nodes, R.n_comms, part_off, P, n, s->parts);
+    note_launch();
+    return build_memberships(R, n, &s->members, st);
+}
+
+// The last tier of one direction: a global table per community, 2
+// min(incidences, |B|) entries; communities go in chunks whose tables fit a
+// bounded scratch (a single table is at most 2^(1+ceil log2 |B|) entries).
+int global_tier(PairArgs a, int dir, i64 nk, cudaStream_t st) {
+    const Direction &d = a.d[dir];
+    i64 *tsz = nullptr, *toff = nullptr;
+    i32 *tables = nullptr;
     unsigned int *tfill = nullptr;
-    unsigned long long *cnt = nullptr, *amax = nullptr;
     int rc = MSCD_OK;
     do {
-        if (n_active == 0) break;
-        if ((rc = dev_alloc(&spill, n_active, st))) break;
-        // spills, big-B count, spills of the block tier, then the launches' work counters
-        if ((rc = dev_alloc(&cnt, 6, st))) break;
-        if ((rc = dev_alloc(&big, B.n_comms, st))) break;
-        if ((rc = dev_alloc(&amax, P, st))) break;
-        if ((rc = cuda_status(cudaMemsetAsync(cnt, 0, 6 * sizeof(unsigned long long), st)))) break;
-        if ((rc = cuda_status(cudaMemsetAsync(amax, 0, (size_t)P * sizeof(unsigned long long), st)))) break;
-        DirArgs a{};
-        a.aptr = A.comm_ptr;
-        a.anodes = A.comm_nodes;
-        a.active = active;
-        a.n_active = n_active;
-        a.bptr = B.comm_ptr;
-        a.mptr = MB.ptr;
-        a.mlist = MB.list;
-        a.acn = PA.cn;
-        a.best = best;
-        a.spill = spill;
-        a.n_spill = cnt;
-        a.next = cnt + 3;
-        pairs_smem<<<(unsigned)std::min<i64>((n_active + NMI_WARPS - 1) / NMI_WARPS, 152 * 6), NMI_WARPS * 32, 0,
-                     st>>>(a); note_launch();
-        active_max_size<<<GB, 256, 0, st>>>(A.comm_ptr, active, n_active, PA.cp, amax); note_launch();
-        list_big<<<GB, 256, 0, st>>>(B.comm_ptr, B.n_comms, PB.cp, PB.cn, amax, big, cnt + 1); note_launch();
-        unsigned long long h[2] = {0, 0};
-        if ((rc = cuda_status(cudaMemcpyAsync(h, cnt, sizeof(h), cudaMemcpyDeviceToHost, st)))) break;
+        if ((rc = dev_alloc(&tsz, nk + 1, st))) break;
+        if ((rc = dev_alloc(&toff, nk + 1, st))) break;
+        spill_sizes<<<GB, 256, 0, st>>>(d.spill2, nk, d, tsz); note_launch();
+        std::vector<i64> hs(nk);
+        if ((rc = cuda_status(cudaMemcpyAsync(hs.data(), tsz, nk * sizeof(i64), cudaMemcpyDeviceToHost, st)))) break;
         if ((rc = cuda_status(cudaStreamSynchronize(st)))) break;
-        i64 nk = (i64)h[0];
-        const i64 *list = spill;
-        if (nk > 0) {
-            // middle tier: one community per CTA with a large shared-memory table
-            if ((rc = dev_alloc(&spill2, nk, st))) break;
-            const size_t bsm = 2 * sizeof(i32) * BLK_TABLE + sizeof(unsigned short) * (BLK_TABLE / 2);
-            if ((rc = cuda_status(cudaFuncSetAttribute(pairs_block, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                       (int)bsm))))
-                break;
-            a.next = cnt + 4;
-            // as many CTAs as fit the SMs' shared memory
-            const i64 per_sm = std::max<i64>(1, (i64)(216 * 1024) / (i64)bsm);
-            pairs_block<<<(unsigned)std::min<i64>(nk, 152 * per_sm), BLK_WARPS * 32, bsm, st>>>(a, spill, nk, spill2,
-                                                                                           cnt + 2);
-            note_launch();
-            unsigned long long h2 = 0;
-            if ((rc = cuda_status(cudaMemcpyAsync(&h2, cnt + 2, sizeof(h2), cudaMemcpyDeviceToHost, st)))) break;
-            if ((rc = cuda_status(cudaStreamSynchronize(st)))) break;
-            nk = (i64)h2;
-            list = spill2;
+        i64 largest = 0, all = 0;
+        for (i64 v : hs) {
+            largest = std::max(largest, v);
+            all += v;
         }
-        if (nk > 0) {
-            // last tier: a global table per community, 2 min(incidences, |B|)
-            // entries; communities go in chunks whose tables fit a bounded
-            // scratch (a single table is at most 2^(1+ceil log2 |B|) entries)
-            if ((rc = dev_alloc(&tsz, nk + 1, st))) break;
-            if ((rc = dev_alloc(&toff, nk + 1, st))) break;
-            spill_sizes<<<GB, 256, 0, st>>>(list, nk, active, A.comm_ptr, A.comm_nodes, MB.cnt, B.n_comms, tsz); note_launch();
-            std::vector<i64> hs(nk);
-            if ((rc = cuda_status(cudaMemcpyAsync(hs.data(), tsz, nk * sizeof(i64), cudaMemcpyDeviceToHost, st)))) break;
-            if ((rc = cuda_status(cudaStreamSynchronize(st)))) break;
-            i64 largest = 0;
-            for (i64 v : hs) largest = std::max(largest, v);
-            size_t fr = 0, tot = 0;
-            cudaMemGetInfo(&fr, &tot);
-            const i64 budget = std::max<i64>(largest, std::min<i64>((i64)1 << 28, (i64)(fr / 8 / (3 * sizeof(i32)))));
-            if ((rc = dev_alloc(&tkey, budget, st))) break;
-            if ((rc = dev_alloc(&tcnt, budget, st))) break;
-            if ((rc = dev_alloc(&tused, budget, st))) break;
-            if ((rc = dev_alloc(&tfill, nk, st))) break;
-            // emptied once; each community empties the buckets it claimed
-            if ((rc = cuda_status(cudaMemsetAsync(tkey, 0xff, budget * sizeof(i32), st)))) break;
-            if ((rc = cuda_status(cudaMemsetAsync(tcnt, 0, budget * sizeof(i32), st)))) break;
-            a.tkey = tkey;
-            a.tcnt = tcnt;
-            a.tused = tused;
-            a.tfill = tfill;
-            a.toff = toff;
-            std::vector<i64> ho;
-            for (i64 r0 = 0; r0 < nk && rc == MSCD_OK;) {
-                ho.assign(1, 0);
-                i64 r1 = r0;
-                while (r1 < nk && ho.back() + hs[r1] <= budget) {
-                    ho.push_back(ho.back() + hs[r1]);
-                    ++r1;
-                }
-                if ((rc = cuda_status(cudaMemcpyAsync(toff, ho.data(), ho.size() * sizeof(i64), cudaMemcpyHostToDevice,
-                                                      st))))
-                    break;
-                if ((rc = cuda_status(cudaMemsetAsync(tfill, 0, (r1 - r0) * sizeof(unsigned int), st)))) break;
-                if ((rc = cuda_status(cudaMemsetAsync(cnt + 5, 0, sizeof(unsigned long long), st)))) break;
-                a.next = cnt + 5;
-                pairs_global<<<(unsigned)std::min<i64>(r1 - r0, 152 * 4), GLB_WARPS * 32, 0, st>>>(a, list + r0,
-                                                                                              r1 - r0);
-                note_launch();
-                // the host offsets are read by the copy before the next chunk rewrites them
-                if ((rc = cuda_status(cudaStreamSynchronize(st)))) break;
-                r0 = r1;
+        size_t fr = 0, tot = 0;
+        cudaMemGetInfo(&fr, &tot);
+        const i64 budget = std::max<i64>(
+            largest, std::min<i64>(all, std::min<i64>((i64)1 << 28, (i64)(fr / 8 / (3 * sizeof(i32))))));
+        if ((rc = dev_alloc(&tables, 3 * budget, st))) break;
+        if ((rc = dev_alloc(&tfill, nk, st))) break;
+        a.tkey = tables;
+        a.tcnt = tables + budget;
+        a.tused = tables + 2 * budget;
+        a.tfill = tfill;
+        a.toff = toff;
+        // emptied once; each community empties the buckets it claimed
+        if ((rc = cuda_status(cudaMemsetAsync(a.tkey, 0xff, budget * sizeof(i32), st)))) break;
+        if ((rc = cuda_status(cudaMemsetAsync(a.tcnt, 0, budget * sizeof(i32), st)))) break;
+        std::vector<i64> ho;
+        for (i64 r0 = 0; r0 < nk && rc == MSCD_OK;) {
+            ho.assign(1, 0);
+            i64 r1 = r0;
+            while (r1 < nk && ho.back() + hs[r1] <= budget) {
+                ho.push_back(ho.back() + hs[r1]);
+                ++r1;
             }
-        }
-        if (h[1] > 0) {
-            // group the candidate B communities by part, in descending size
-            // inside a part (host sort: they are few)
-            const i64 nb = (i64)h[1];
-            std::vector<i32> hb(nb), hp(nb), sorted(nb);
-            std::vector<i64> hsz(nb), order(nb);
-            std::vector<i64> boff(P + 1, 0);
-            if ((rc = dev_alloc(&bpart, nb, st))) break;
-            if ((rc = dev_alloc(&bsize, nb, st))) break;
-            if ((rc = dev_alloc(&dboff, P + 1, st))) break;
-            gather_parts<<<GB, 256, 0, st>>>(big, nb, PB.cp, B.comm_ptr, bpart, bsize); note_launch();
-            if ((rc = cuda_status(cudaMemcpyAsync(hb.data(), big, nb * sizeof(i32), cudaMemcpyDeviceToHost, st))))
-                break;
-            if ((rc = cuda_status(cudaMemcpyAsync(hp.data(), bpart, nb * sizeof(i32), cudaMemcpyDeviceToHost, st))))
-                break;
-            if ((rc = cuda_status(cudaMemcpyAsync(hsz.data(), bsize, nb * sizeof(i64), cudaMemcpyDeviceToHost, st))))
-                break;
-            if ((rc = cuda_status(cudaStreamSynchronize(st)))) break;
-            for (i64 i = 0; i < nb; ++i) order[i] = i;
-            std::sort(order.begin(), order.end(), [&](i64 x, i64 y) {
-                if (hp[x] != hp[y]) return hp[x] < hp[y];
-                if (hsz[x] != hsz[y]) return hsz[x] > hsz[y];
-                return hb[x] < hb[y];
-            });
-            for (i64 i = 0; i < nb; ++i) {
-                sorted[i] = hb[order[i]];
-                boff[hp[i] + 1]++;
-            }
-            for (int32_t q = 0; q < P; ++q) boff[q + 1] += boff[q];
-            if ((rc = cuda_status(cudaMemcpyAsync(big, sorted.data(), nb * sizeof(i32), cudaMemcpyHostToDevice, st))))
-                break;
-            if ((rc = cuda_status(cudaMemcpyAsync(dboff, boff.data(), (P + 1) * sizeof(i64), cudaMemcpyHostToDevice,
+            if ((rc = cuda_status(cudaMemcpyAsync(toff, ho.data(), ho.size() * sizeof(i64), cudaMemcpyHostToDevice,
                                                   st))))
                 break;
-            disjoint_pairs<<<GB, 256, 0, st>>>(A.comm_ptr, A.comm_nodes, active, n_active, B.comm_ptr, B.comm_nodes,
-                                               big, dboff, PA.cp, PA.cn, best); note_launch();
-            if ((rc = cuda_status(cudaStreamSynchronize(st)))) break;  // host vectors outlive the copies
+            if ((rc = cuda_status(cudaMemsetAsync(tfill, 0, (r1 - r0) * sizeof(unsigned int), st)))) break;
+            if ((rc = cuda_status(cudaMemsetAsync(a.next_global, 0, sizeof(unsigned long long), st)))) break;
+            pairs_global<<<(unsigned)std::min<i64>(r1 - r0, 152 * 4), GLB_WARPS * 32, 0, st>>>(a, dir, d.spill2 + r0,
+                                                                                              r1 - r0);
+            note_launch();
+            // the host offsets are read by the copy before the next chunk rewrites them
+            if ((rc = cuda_status(cudaStreamSynchronize(st)))) break;
+            r0 = r1;
         }
     } while (0);
-    cudaFreeAsync(spill, st);
-    if (spill2) cudaFreeAsync(spill2, st);
-    cudaFreeAsync(cnt, st);
-    cudaFreeAsync(big, st);
-    if (tsz) cudaFreeAsync(tsz, st);
-    if (toff) cudaFreeAsync(toff, st);
-    if (tkey) cudaFreeAsync(tkey, st);
-    if (tcnt) cudaFreeAsync(tcnt, st);
-    if (tused) cudaFreeAsync(tused, st);
-    if (tfill) cudaFreeAsync(tfill, st);
-    if (bpart) cudaFreeAsync(bpart, st);
-    if (bsize) cudaFreeAsync(bsize, st);
-    if (dboff) cudaFreeAsync(dboff, st);
-    if (amax) cudaFreeAsync(amax, st);
+    cudaFreeAsync(tsz, st);
+    cudaFreeAsync(toff, st);
+    cudaFreeAsync(tables, st);
+    cudaFreeAsync(tfill, st);
+    return rc;
+}
+
+// One pair of scales into acc (6 P words, zero).  Waits for the stream only
+// where a community may meet more partners than a CTA's table holds.
+int pair_terms(const ScaleResult &X, const ScaleResult &Y, const ScaleData &DX, const ScaleData &DY, int32_t P,
+               const double *tab, unsigned long long *acc, cudaStream_t st) {
+    const i64 C[2] = {X.n_comms, Y.n_comms};
+    i64 T = 2;
+    while (T < 2 * C[1]) T <<= 1;
+    // one allocation: what starts as zero first
+    enum { N_ACTIVE = 0, N_SPILL = 2, N_SPILL2 = 4, NEXT_WARP = 6, NEXT_BLOCK, NEXT_GLOBAL, COUNTERS };
+    size_t at = 0;
+    auto room = [&](size_t bytes) {
+        const size_t o = at;
+        at += (bytes + 15) & ~(size_t)15;
+        return o;
+    };
+    const size_t o_cnt = room(COUNTERS * 8), o_part = room(8 * (size_t)P * 8), o_tkey = room((size_t)T * 8);
+    const size_t o_zero[2] = {room((size_t)C[0]), room((size_t)C[1])};
+    const size_t zeroed = at;
+    const size_t o_tval = room((size_t)T * 4), o_boff = room(2 * ((size_t)P + 1) * 8);
+    size_t o_best[2], o_act[2], o_big[2], o_sp[2], o_sp2[2];
+    for (int i = 0; i < 2; ++i) {
+        o_best[i] = room((size_t)C[i] * 8);
+        o_act[i] = room((size_t)C[i] * 4);
+        o_big[i] = room((size_t)C[1 - i] * 4);
+        o_sp[i] = room((size_t)C[i] * 8);
+        o_sp2[i] = room((size_t)C[i] * 8);
+    }
+    unsigned char *mem = nullptr;
+    int rc = dev_alloc(&mem, (i64)at, st);
+    if (rc) return rc;
+    unsigned long long *cnt = (unsigned long long *)(mem + o_cnt), *part = (unsigned long long *)(mem + o_part);
+    PairArgs a{};
+    a.P = P;
+    a.tab = tab;
+    a.next_warp = cnt + NEXT_WARP;
+    a.next_block = cnt + NEXT_BLOCK;
+    a.next_global = cnt + NEXT_GLOBAL;
+    for (int i = 0; i < 2; ++i) {
+        const ScaleResult &A = i ? Y : X, &B = i ? X : Y;
+        const ScaleData &DA = i ? DY : DX, &DB = i ? DX : DY;
+        Direction &d = a.d[i];
+        d.aptr = A.comm_ptr;
+        d.anodes = A.comm_nodes;
+        d.CA = A.n_comms;
+        d.ap = DA.parts;
+        d.zero = mem + o_zero[i];
+        d.active = (i32 *)(mem + o_act[i]);
+        d.n_active = cnt + N_ACTIVE + i;
+        d.best = (unsigned long long *)(mem + o_best[i]);
+        d.amax = part + (size_t)(4 * i) * P;
+        d.bmax = part + (size_t)(4 * i + 1) * P;
+        d.bcount = part + (size_t)(4 * i + 2) * P;
+        d.bfill = part + (size_t)(4 * i + 3) * P;
+        d.bptr = B.comm_ptr;
+        d.CB = B.n_comms;
+        d.bp = DB.parts;
+        d.mcnt = DB.members.cnt;
+        d.mptr = DB.members.ptr;
+        d.mlist = DB.members.list;
+        d.big = (i32 *)(mem + o_big[i]);
+        d.boff = (i64 *)(mem + o_boff) + (size_t)i * (P + 1);
+        d.spill = (i64 *)(mem + o_sp[i]);
+        d.spill2 = (i64 *)(mem + o_sp2[i]);
+        d.n_spill = cnt + N_SPILL + i;
+        d.n_spill2 = cnt + N_SPILL2 + i;
+    }
+    u64 *tkey = (u64 *)(mem + o_tkey);
+    i32 *tval = (i32 *)(mem + o_tval);
+    const i64 most = std::max(C[0], C[1]);
+    const dim3 both(grid_of(most), 2);
+    do {
+        if ((rc = cuda_status(cudaMemsetAsync(mem, 0, zeroed, st)))) break;
+        // identical communities
+        hash_insert<<<grid_of(C[1]), 256, 0, st>>>(Y.comm_hash, C[1], tkey, tval, T - 1); note_launch();
+        match_identical<<<grid_of(32 * C[0]), 256, 0, st>>>(X.comm_ptr, X.comm_nodes, X.comm_hash, C[0], Y.comm_ptr,
+                                                            Y.comm_nodes, tkey, tval, T - 1, mem + o_zero[0],
+                                                            mem + o_zero[1]); note_launch();
+        init_best<<<both, 256, 0, st>>>(a); note_launch();
+        list_big<<<both, 256, 0, st>>>(a, 0); note_launch();
+        big_offsets<<<dim3(1, 2), 32, 0, st>>>(a); note_launch();
+        list_big<<<both, 256, 0, st>>>(a, 1); note_launch();
+        pairs_warp<<<(unsigned)std::min<i64>((C[0] + C[1] + NMI_WARPS - 1) / NMI_WARPS, 152 * 5), NMI_WARPS * 32, 0,
+                     st>>>(a); note_launch();
+        const size_t bsm = 2 * sizeof(i32) * BLK_TABLE + sizeof(unsigned short) * (BLK_TABLE / 2);
+        if ((rc = cuda_status(cudaFuncSetAttribute(pairs_block, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)bsm))))
+            break;
+        pairs_block<<<(unsigned)std::min<i64>(C[0] + C[1], 152 * 3), BLK_WARPS * 32, bsm, st>>>(a); note_launch();
+        if (most > BLK_TABLE / 2) {
+            unsigned long long h[2] = {0, 0};
+            if ((rc = cuda_status(cudaMemcpyAsync(h, cnt + N_SPILL2, sizeof(h), cudaMemcpyDeviceToHost, st)))) break;
+            if ((rc = cuda_status(cudaStreamSynchronize(st)))) break;
+            for (int i = 0; i < 2 && rc == MSCD_OK; ++i)
+                if (h[i]) rc = global_tier(a, i, (i64)h[i], st);
+            if (rc) break;
+        }
+        normalise_sum<<<both, 256, 0, st>>>(a, acc); note_launch();
+        rc = cuda_status(cudaGetLastError());
+    } while (0);
+    cudaFreeAsync(mem, st);
     return rc;
 }
 
 }  // namespace
 
-int nmi_between(const ScaleResult &X, const ScaleResult &Y, i64 n, const i64 *part_off, int32_t n_parts, double *nmi,
-                cudaStream_t st) {
-    const i64 CX = X.n_comms, CY = Y.n_comms;
-    const int32_t P = part_off ? n_parts : 1;
-    for (int32_t p = 0; p < P; ++p) nmi[p] = __builtin_nan("");
-    if (CX <= 0 || CY <= 0 || n <= 0) return MSCD_OK;
-    u64 *tkey = nullptr;
-    i32 *tval = nullptr, *actX = nullptr, *actY = nullptr;
-    unsigned char *zeroX = nullptr, *zeroY = nullptr;
-    unsigned long long *bestX = nullptr, *bestY = nullptr, *cnt = nullptr, *acc = nullptr;
-    CommParts PX, PY;
-    Memberships MX, MY;
+int nmi_chain(const ScaleResult *sc, int32_t S, i64 n, const i64 *part_off, int32_t n_parts, double *nmi,
+              cudaStream_t st) {
+    const int32_t P = part_off ? n_parts : 1, pairs = std::max(S - 1, 0);
+    for (i64 i = 0; i < (i64)pairs * P; ++i) nmi[i] = __builtin_nan("");
+    if (pairs == 0 || n <= 0) return MSCD_OK;
+    double *tab = nullptr;
+    unsigned long long *acc = nullptr;
+    ScaleData data[2];  // of scales s and s + 1, by parity
+    const size_t words = 6 * (size_t)P;
+    std::vector<unsigned long long> h(words * pairs);
     int rc = MSCD_OK;
-    i64 T = 2;
-    while (T < 2 * CY) T <<= 1;
-    // acc: per part, X's 128-bit sum, Y's 128-bit sum, X's count, Y's count
-    const i64 acc_words = 6 * (i64)P;
     do {
-        if ((rc = dev_alloc(&tkey, T, st))) break;
-        if ((rc = dev_alloc(&tval, T, st))) break;
-        if ((rc = dev_alloc(&zeroX, CX, st))) break;
-        if ((rc = dev_alloc(&zeroY, CY, st))) break;
-        if ((rc = dev_alloc(&bestX, CX, st))) break;
-        if ((rc = dev_alloc(&bestY, CY, st))) break;
-        if ((rc = dev_alloc(&actX, CX, st))) break;
-        if ((rc = dev_alloc(&actY, CY, st))) break;
-        if ((rc = dev_alloc(&PX.cp, CX, st))) break;
-        if ((rc = dev_alloc(&PX.cn, CX, st))) break;
-        if ((rc = dev_alloc(&PY.cp, CY, st))) break;
-        if ((rc = dev_alloc(&PY.cn, CY, st))) break;
-        if ((rc = dev_alloc(&cnt, 2, st))) break;
-        if ((rc = dev_alloc(&acc, acc_words, st))) break;
-        if ((rc = cuda_status(cudaMemsetAsync(tkey, 0, T * sizeof(u64), st)))) break;
-        if ((rc = cuda_status(cudaMemsetAsync(zeroX, 0, CX, st)))) break;
-        if ((rc = cuda_status(cudaMemsetAsync(zeroY, 0, CY, st)))) break;
-        if ((rc = cuda_status(cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned long long), st)))) break;
-        if ((rc = cuda_status(cudaMemsetAsync(acc, 0, acc_words * sizeof(unsigned long long), st)))) break;
-        comm_parts<<<GB, 256, 0, st>>>(X.comm_ptr, X.comm_nodes, CX, part_off, P, n, PX.cp, PX.cn); note_launch();
-        comm_parts<<<GB, 256, 0, st>>>(Y.comm_ptr, Y.comm_nodes, CY, part_off, P, n, PY.cp, PY.cn); note_launch();
-        // identical communities
-        hash_insert<<<GB, 256, 0, st>>>(Y.comm_hash, CY, tkey, tval, T - 1); note_launch();
-        match_identical<<<GB, 256, 0, st>>>(X.comm_ptr, X.comm_nodes, X.comm_hash, CX, Y.comm_ptr, Y.comm_nodes, tkey,
-                                            tval, T - 1, zeroX, zeroY); note_launch();
-        init_best<<<GB, 256, 0, st>>>(X.comm_ptr, CX, PX.cn, zeroX, bestX, actX, cnt); note_launch();
-        init_best<<<GB, 256, 0, st>>>(Y.comm_ptr, CY, PY.cn, zeroY, bestY, actY, cnt + 1); note_launch();
-        unsigned long long na[2] = {0, 0};
-        if ((rc = cuda_status(cudaMemcpyAsync(na, cnt, sizeof(na), cudaMemcpyDeviceToHost, st)))) break;
-        if ((rc = cuda_status(cudaStreamSynchronize(st)))) break;
-        // H(X_k|Y) for the X communities without an identical partner
-        if (na[0] > 0) {
-            if ((rc = build_memberships(Y, n, &MY, st))) break;
-            if ((rc = one_direction(X, Y, MY, PX, PY, P, actX, (i64)na[0], bestX, st))) break;
+        if (n <= TERMS_MAX) {
+            if ((rc = dev_alloc(&tab, n + P, st))) break;
+            fill_terms<<<grid_of(n + P), 256, 0, st>>>(part_off, P, n, tab); note_launch();
         }
-        // H(Y_l|X) likewise
-        if (na[1] > 0) {
-            if ((rc = build_memberships(X, n, &MX, st))) break;
-            if ((rc = one_direction(Y, X, MX, PY, PX, P, actY, (i64)na[1], bestY, st))) break;
+        if ((rc = dev_alloc(&acc, (i64)h.size(), st))) break;
+        if ((rc = cuda_status(cudaMemsetAsync(acc, 0, h.size() * sizeof(acc[0]), st)))) break;
+        for (int32_t s = 0; s < S && rc == MSCD_OK; ++s) {
+            free_scale(&data[s & 1], st);
+            if (sc[s].n_comms <= 0) continue;
+            if ((rc = build_scale(sc[s], n, part_off, P, &data[s & 1], st))) break;
+            if (s > 0 && sc[s - 1].n_comms > 0)
+                rc = pair_terms(sc[s - 1], sc[s], data[(s - 1) & 1], data[s & 1], P, tab, acc + words * (s - 1), st);
         }
-        normalise_sum<<<GB, 256, 0, st>>>(X.comm_ptr, CX, PX.cn, PX.cp, bestX, acc, acc + 4 * P); note_launch();
-        normalise_sum<<<GB, 256, 0, st>>>(Y.comm_ptr, CY, PY.cn, PY.cp, bestY, acc + 2 * P, acc + 5 * P);
-        note_launch();
-        std::vector<unsigned long long> h(acc_words);
-        if ((rc = cuda_status(cudaMemcpyAsync(h.data(), acc, acc_words * sizeof(unsigned long long),
-                                              cudaMemcpyDeviceToHost, st))))
+        if (rc) break;
+        if ((rc = cuda_status(cudaMemcpyAsync(h.data(), acc, h.size() * sizeof(acc[0]), cudaMemcpyDeviceToHost, st))))
             break;
         if ((rc = cuda_status(cudaStreamSynchronize(st)))) break;
-        for (int32_t p = 0; p < P; ++p) {
-            const unsigned long long cx = h[4 * P + p], cy = h[5 * P + p];
-            if (!cx || !cy) continue;  // a part without communities at one of the scales
-            const double sx = (double)h[2 * p + 1] * 4.0 + (double)h[2 * p] * 0x1p-62;
-            const double sy = (double)h[2 * P + 2 * p + 1] * 4.0 + (double)h[2 * P + 2 * p] * 0x1p-62;
-            nmi[p] = 1.0 - 0.5 * (sx / (double)cx + sy / (double)cy);
-        }
+        for (int32_t s = 0; s < pairs; ++s)
+            for (int32_t p = 0; p < P; ++p) {
+                const unsigned long long *w = h.data() + words * s;
+                const unsigned long long cx = w[4 * (size_t)P + p], cy = w[5 * (size_t)P + p];
+                if (!cx || !cy) continue;  // a part without communities at one of the scales
+                const double sx = (double)w[2 * p + 1] * 4.0 + (double)w[2 * p] * 0x1p-62;
+                const double sy = (double)w[2 * (size_t)P + 2 * p + 1] * 4.0 + (double)w[2 * (size_t)P + 2 * p] * 0x1p-62;
+                nmi[(size_t)s * P + p] = 1.0 - 0.5 * (sx / (double)cx + sy / (double)cy);
+            }
     } while (0);
-    free_memberships(&MX, st);
-    free_memberships(&MY, st);
-    cudaFreeAsync(tkey, st);
-    cudaFreeAsync(tval, st);
-    cudaFreeAsync(zeroX, st);
-    cudaFreeAsync(zeroY, st);
-    cudaFreeAsync(bestX, st);
-    cudaFreeAsync(bestY, st);
-    cudaFreeAsync(actX, st);
-    cudaFreeAsync(actY, st);
-    cudaFreeAsync(PX.cp, st);
-    cudaFreeAsync(PX.cn, st);
-    cudaFreeAsync(PY.cp, st);
-    cudaFreeAsync(PY.cn, st);
-    cudaFreeAsync(cnt, st);
+    for (auto &x : data) free_scale(&x, st);
+    cudaFreeAsync(tab, st);
     cudaFreeAsync(acc, st);
+    if (rc) cudaStreamSynchronize(st);
     return rc != MSCD_OK ? rc : cuda_status(cudaGetLastError());
 }
 
@@ -906,8 +1012,8 @@ extern "C" int mscd_nmi_covers(mscd_ctx *ctx, int64_t n, const int64_t *ptr_a, c
     ScaleResult A, B;
     int rc = cover_to_device(ptr_a, nodes_a, n_a, n, &A, st);
     if (!rc) rc = cover_to_device(ptr_b, nodes_b, n_b, n, &B, st);
-    if (!rc) rc = nmi_between(A, B, n, nullptr, 1, nmi, st);
-    if (!rc) rc = cuda_status(cudaStreamSynchronize(st));
+    ScaleResult two[2] = {A, B};
+    if (!rc) rc = nmi_chain(two, 2, n, nullptr, 1, nmi, st);
     scale_result_free(&A);
     scale_result_free(&B);
     return rc;
