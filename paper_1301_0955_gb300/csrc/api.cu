@@ -24,9 +24,9 @@ namespace {
 
 struct GraphRec {
     bool live = false;
+    void *block = nullptr;  // a loaded graph: one allocation that the arrays below lie in (a union: their own)
     i64 *rp = nullptr;
     i32 *col = nullptr;
-    float *w = nullptr;
     i64 *wfx = nullptr, *k = nullptr;
     float *logk = nullptr;
     DevGraph g;
@@ -180,12 +180,14 @@ void free_run(mscd_ctx *c) {
 }
 
 void free_graph(GraphRec &g) {
-    cudaFree(g.rp);
-    cudaFree(g.col);
-    cudaFree(g.w);
-    cudaFree(g.wfx);
-    cudaFree(g.k);
-    cudaFree(g.logk);
+    cudaFree(g.block);
+    if (!g.block) {
+        cudaFree(g.rp);
+        cudaFree(g.col);
+        cudaFree(g.wfx);
+        cudaFree(g.k);
+        cudaFree(g.logk);
+    }
     cudaFree(g.part_off);
     g = GraphRec{};
 }
@@ -341,25 +343,41 @@ int mscd_graph_load_csr(mscd_ctx *c, int64_t n, const int64_t *row_ptr, const in
     else nnz = row_ptr[n];
     if (nnz < 0 || (nnz > 0 && !col)) return MSCD_EINVAL;
     GraphRec g;
+    float *wdev = nullptr;  // host weights on the device (device weights are read where they are)
     int rc = MSCD_OK;
     do {
-        if ((rc = cuda_status(cudaMalloc((void **)&g.rp, (size_t)(n + 1) * sizeof(i64))))) break;
-        if ((rc = cuda_status(cudaMalloc((void **)&g.col, (size_t)std::max<i64>(nnz, 1) * sizeof(i32))))) break;
+        // one allocation and one release per graph: each costs some 70 us
+        size_t at = 0;
+        auto room = [&](size_t bytes) {
+            const size_t o = at;
+            at += (bytes + 255) & ~(size_t)255;
+            return o;
+        };
+        const size_t m = (size_t)std::max<i64>(nnz, 1), rows = (size_t)std::max<i64>(n, 1);
+        const size_t o_rp = room((size_t)(n + 1) * sizeof(i64)), o_k = room(rows * sizeof(i64)),
+                     o_logk = room(rows * sizeof(float)), o_col = room(m * sizeof(i32)),
+                     o_wfx = room(w ? m * sizeof(i64) : 0);
+        if ((rc = cuda_status(cudaMalloc(&g.block, at)))) break;
+        unsigned char *base = (unsigned char *)g.block;
+        g.rp = (i64 *)(base + o_rp);
+        g.k = (i64 *)(base + o_k);
+        g.logk = (float *)(base + o_logk);
+        g.col = (i32 *)(base + o_col);
+        g.wfx = w ? (i64 *)(base + o_wfx) : nullptr;
         if ((rc = cuda_status(cudaMemcpyAsync(g.rp, row_ptr, (size_t)(n + 1) * sizeof(i64), kind, st)))) break;
         if (nnz > 0 && (rc = cuda_status(cudaMemcpyAsync(g.col, col, (size_t)nnz * sizeof(i32), kind, st)))) break;
-        if (w) {
-            if ((rc = cuda_status(cudaMalloc((void **)&g.w, (size_t)std::max<i64>(nnz, 1) * sizeof(float))))) break;
-            if (nnz > 0 && (rc = cuda_status(cudaMemcpyAsync(g.w, w, (size_t)nnz * sizeof(float), kind, st)))) break;
+        if (w && !dev) {
+            if ((rc = cuda_status(cudaMallocAsync((void **)&wdev, m * sizeof(float), st)))) break;
+            if (nnz > 0 && (rc = cuda_status(cudaMemcpyAsync(wdev, w, (size_t)nnz * sizeof(float), kind, st)))) break;
         }
-        rc = graph_prepare(n, g.rp, g.col, g.w, &g.g, &g.wfx, &g.k, &g.logk, st);
+        rc = graph_prepare(n, nnz, g.rp, g.col, w && !dev ? wdev : w, g.wfx, g.k, g.logk, &g.g, st);
     } while (0);
+    if (wdev) cudaFreeAsync(wdev, st);
     if (rc != MSCD_OK) {
         cudaStreamSynchronize(st);
         free_graph(g);
         return rc;
     }
-    cudaFree(g.w);  // the exact fixed-point copy replaces it
-    g.w = nullptr;
     g.live = true;
     g.parts = {0, n};
     g.max_part_n = n;

@@ -50,9 +50,10 @@ int scan_exclusive_i64(const i64 *in, i64 *out, i64 n, i64 *total_dev, cudaStrea
 struct mscd_ctx;
 bool ctx_graph(mscd_ctx *c, int32_t graph_id, DevGraph *g, int *device);
 
-// Graph preparation (checks, exact weights, degrees, log degrees).
-int graph_prepare(i64 n, const i64 *rp_dev, const i32 *col_dev, const float *w_dev, DevGraph *g, i64 **wfx_out,
-                  i64 **k_out, float **logk_out, cudaStream_t st);
+// Graph preparation: checks, exact weights (into wfx, weighted graphs only),
+// degrees and their logarithms (into k and logk).
+int graph_prepare(i64 n, i64 nnz, const i64 *rp, const i32 *col, const float *w, i64 *wfx, i64 *k, float *logk,
+                  DevGraph *g, cudaStream_t st);
 
 // Disjoint union of graphs as one graph (node ids of part p shifted by the
 // nodes of the parts before it); node_off gets the n_parts+1 offsets.  All parts

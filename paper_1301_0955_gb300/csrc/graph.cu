@@ -27,15 +27,17 @@ enum : u32 {
 struct PrepState {
     u32 mask;
     int min_lowbit;
-    unsigned long long total;  // exact volume (valid while total_d < 2^63)
-    double total_d;            // coarse volume, guards against wrap-around
-    unsigned long long kmax;   // largest degree
+    unsigned long long total;      // exact volume (valid while total_d < 2^63)
+    double total_d;                // coarse volume (within 1%), guards against wrap-around
+    unsigned long long kmax;       // largest degree
+    unsigned long long below;      // entries with a smaller column than their row, minus those with a larger one
 };
 
-__global__ void check_row_ptr(const i64 *rp, i64 n, PrepState *ps) {
+__global__ void check_row_ptr(const i64 *rp, i64 n, i64 nnz, PrepState *ps) {
     i64 u = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (u > n) return;
     bool bad = (u == 0) ? (rp[0] != 0) : (rp[u] < rp[u - 1]);
+    if (u == n) bad = bad || rp[n] != nnz;
     if (bad) atomicOr(&ps->mask, CAT_STRUCT);
 }
 
@@ -52,11 +54,18 @@ __device__ __forceinline__ int f32_lowbit(float w, u32 *odd) {
 
 // Warp per row: per-entry checks (column range, weight, self-loop, order,
 // duplicate, symmetric partner with the same weight) and the smallest lowbit.
+// Only entries above the diagonal look for their partner: with rows sorted and
+// free of repeats (else an earlier category is reported) the partners are
+// distinct entries below it, so if there are as many entries below as above
+// none is left over.  The look-ups (a binary search each) are what the kernel
+// takes its time for: half of them, 969 -> 600 us for 27 million entries.
 __global__ void check_entries(const i64 *rp, const i32 *col, const float *w, i64 n, PrepState *ps) {
+    if (*(volatile u32 *)&ps->mask) return;  // the row pointers cannot be followed
     const int lane = threadIdx.x & 31;
     const i64 warps = (i64)gridDim.x * (blockDim.x >> 5);
     u32 mask = 0;
     int lowbit = INT32_MAX;
+    i64 below = 0;
     for (i64 u = (i64)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); u < n; u += warps) {
         const i64 rs = rp[u], re = rp[u + 1];
         for (i64 e = rs + lane; e < re; e += 32) {
@@ -80,76 +89,139 @@ __global__ void check_entries(const i64 *rp, const i32 *col, const float *w, i64
                 if (c < p) mask |= CAT_UNSORTED;
                 else if (c == p) mask |= CAT_DUP;
             }
+            below += (i64)c < u ? 1 : -1;
+            if ((i64)c <= u) continue;
             // partner entry c -> u by binary search in row c
-            i64 lo = rp[c], hi = rp[(i64)c + 1];
-            while (lo < hi) {
-                i64 mid = lo + ((hi - lo) >> 1);
-                if ((i64)col[mid] < u) lo = mid + 1;
-                else hi = mid;
+            i64 lo = rp[c];
+            const i64 end = rp[(i64)c + 1];
+            for (int len = (int)min(end - lo, (i64)INT32_MAX); len > 0;) {
+                const int half = len >> 1;
+                if ((i64)col[lo + half] < u) {
+                    lo += half + 1;
+                    len -= half + 1;
+                } else {
+                    len = half;
+                }
             }
-            if (lo >= rp[(i64)c + 1] || (i64)col[lo] != u) mask |= CAT_NOTSYM;
+            if (lo >= end || (i64)col[lo] != u) mask |= CAT_NOTSYM;
             else if (w && !(w[lo] == we)) mask |= CAT_NOTSYM;
         }
     }
     mask = __reduce_or_sync(FULL_MASK, mask);
     lowbit = __reduce_min_sync(FULL_MASK, lowbit);
+    for (int o = 16; o; o >>= 1) below += __shfl_xor_sync(FULL_MASK, below, o);
+    // one set of global atomics per block (they all meet on one address)
+    __shared__ u32 bmask;
+    __shared__ int blow;
+    __shared__ unsigned long long bbelow;
+    if (threadIdx.x == 0) {
+        bmask = 0;
+        blow = INT32_MAX;
+        bbelow = 0;
+    }
+    __syncthreads();
     if (lane == 0) {
-        if (mask) atomicOr(&ps->mask, mask);
-        if (lowbit != INT32_MAX) atomicMin(&ps->min_lowbit, lowbit);
+        if (mask) atomicOr(&bmask, mask);
+        atomicMin(&blow, lowbit);
+        atomicAdd(&bbelow, (unsigned long long)below);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (bmask) atomicOr(&ps->mask, bmask);
+        if (blow != INT32_MAX) atomicMin(&ps->min_lowbit, blow);
+        if (bbelow) atomicAdd(&ps->below, bbelow);
     }
 }
 
-__global__ void fixed_weights(const float *w, i64 nnz, int ue, i64 *wfx, PrepState *ps) {
-    for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < nnz; e += (i64)gridDim.x * blockDim.x) {
-        u32 odd;
-        int sh = f32_lowbit(w[e], &odd) - ue;  // >= 0
-        int len = 32 - __clz((int)odd);
-        bool ok = (odd == 1u) ? (sh <= 62) : (len + sh <= 62);
-        if (!ok) {
-            atomicOr(&ps->mask, CAT_RANGE);
-            wfx[e] = 0;
-        } else {
-            wfx[e] = (i64)odd << sh;
-        }
+// The volume, the coarse volume and the largest degree of a block's rows: one
+// set of global atomics per block (they all meet on one address).
+__device__ __forceinline__ void add_totals(unsigned long long tot, float tot_f, unsigned long long kmax, PrepState *ps) {
+    __shared__ unsigned long long btot, bkmax;
+    __shared__ float btot_f;
+    if (threadIdx.x == 0) {
+        btot = bkmax = 0;
+        btot_f = 0.0f;
+    }
+    __syncthreads();
+    for (int o = 16; o; o >>= 1) {
+        tot += __shfl_xor_sync(FULL_MASK, tot, o);
+        tot_f += __shfl_xor_sync(FULL_MASK, tot_f, o);
+        kmax = max(kmax, __shfl_xor_sync(FULL_MASK, kmax, o));
+    }
+    if ((threadIdx.x & 31) == 0) {
+        atomicAdd(&btot, tot);
+        atomicAdd(&btot_f, tot_f);
+        atomicMax(&bkmax, kmax);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        atomicAdd(&ps->total, btot);
+        atomicAdd(&ps->total_d, (double)btot_f);
+        atomicMax(&ps->kmax, bkmax);
     }
 }
 
-// Warp per row: k_u = sum of weights (exact), log k_u, and the volume.
-__global__ void degrees(const i64 *rp, const i64 *wfx, i64 n, i64 *k, float *logk, PrepState *ps) {
-    const int lane = threadIdx.x & 31;
-    const i64 warps = (i64)gridDim.x * (blockDim.x >> 5);
+// Unweighted: thread per row, k_u = its entries.
+__global__ void degrees(const i64 *rp, i64 n, i64 *k, float *logk, PrepState *ps) {
+    if (*(volatile u32 *)&ps->mask) return;
     unsigned long long tot = 0, kmax = 0;
-    double tot_d = 0.0;
-    for (i64 u = (i64)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); u < n; u += warps) {
-        const i64 rs = rp[u], re = rp[u + 1];
+    for (i64 u = (i64)blockIdx.x * blockDim.x + threadIdx.x; u < n; u += (i64)gridDim.x * blockDim.x) {
+        const i64 s = rp[u + 1] - rp[u];
+        k[u] = s;
+        logk[u] = s ? log2f((float)s) : 0.0f;
+        tot += (unsigned long long)s;
+        kmax = max(kmax, (unsigned long long)s);
+    }
+    add_totals(tot, (float)tot, kmax, ps);
+}
+
+// Weighted: half a warp per row writes the exact weights and sums them in the
+// same pass, k_u and log2 k_u.  A sum that might not fit 64 bits (binary32
+// guard, within 1%) is out of range whatever it is.  Bound by the 12 bytes an
+// entry moves: 170 us for 27 million, 69 + 622 us as a pass for the
+// weights and one for the sums with a binary64 guard.
+__global__ void weighted_degrees(const i64 *rp, const float *w, i64 n, i64 *wfx, i64 *k, float *logk, PrepState *ps) {
+    if (*(volatile u32 *)&ps->mask) return;
+    constexpr int ROW = 16;
+    const int lane = threadIdx.x & (ROW - 1);
+    const int ue = *(volatile int *)&ps->min_lowbit;
+    const i64 rows = (i64)gridDim.x * (blockDim.x / ROW);
+    const i64 steps = (n + rows - 1) / rows;
+    unsigned long long tot = 0, kmax = 0;
+    float tot_f = 0.0f;
+    u32 mask = 0;
+    i64 u = (i64)blockIdx.x * (blockDim.x / ROW) + threadIdx.x / ROW;
+    for (i64 step = 0; step < steps; ++step, u += rows) {
         unsigned long long s = 0;
-        double sd = 0.0;
-        if (wfx) {
-            for (i64 e = rs + lane; e < re; e += 32) {
-                s += (unsigned long long)wfx[e];
-                sd += (double)wfx[e];
-            }
-            for (int o = 16; o; o >>= 1) {
-                s += __shfl_xor_sync(FULL_MASK, s, o);
-                sd += __shfl_xor_sync(FULL_MASK, sd, o);
-            }
-        } else {
-            s = (unsigned long long)(re - rs);
-            sd = (double)(re - rs);
+        float f = 0.0f;
+        const i64 re = u < n ? rp[u + 1] : 0;
+        for (i64 e = (u < n ? rp[u] : 0) + lane; e < re; e += ROW) {
+            const float x = w[e];
+            u32 odd;
+            const int sh = f32_lowbit(x, &odd) - ue;  // >= 0
+            const int len = 32 - __clz((int)odd);
+            i64 v = 0;
+            if ((odd == 1u) ? (sh <= 62) : (len + sh <= 62)) v = (i64)odd << sh;
+            else mask |= CAT_RANGE;
+            wfx[e] = v;
+            s += (unsigned long long)v;
+            f += (float)v;
         }
-        if (lane == 0) {
+#pragma unroll
+        for (int o = ROW / 2; o; o >>= 1) {
+            s += __shfl_xor_sync(FULL_MASK, s, o);
+            f += __shfl_xor_sync(FULL_MASK, f, o);
+        }
+        if (lane == 0 && u < n) {
             k[u] = (i64)s;
             logk[u] = s ? log2f((float)(i64)s) : 0.0f;
             tot += s;
-            kmax = s > kmax ? s : kmax;
-            tot_d += sd;
+            tot_f += f;
+            kmax = max(kmax, s);
         }
     }
-    if (lane == 0) {
-        atomicAdd(&ps->total, tot);
-        atomicAdd(&ps->total_d, tot_d);
-        atomicMax(&ps->kmax, kmax);
-    }
+    if (mask) atomicOr(&ps->mask, mask);
+    add_totals(tot, tot_f, kmax, ps);
 }
 
 int first_category(u32 mask) {
@@ -165,64 +237,47 @@ int first_category(u32 mask) {
 
 }  // namespace
 
-int graph_prepare(i64 n, const i64 *rp, const i32 *col, const float *w, DevGraph *g, i64 **wfx_out, i64 **k_out,
-                  float **logk_out, cudaStream_t st) {
-    *wfx_out = nullptr;
-    *k_out = nullptr;
-    *logk_out = nullptr;
+int graph_prepare(i64 n, i64 nnz, const i64 *rp, const i32 *col, const float *w, i64 *wfx, i64 *k, float *logk,
+                  DevGraph *g, cudaStream_t st) {
     PrepState *ps = nullptr;
-    PrepState init{0u, INT32_MAX, 0ull, 0.0, 0ull};
+    const PrepState init{0u, INT32_MAX, 0ull, 0.0, 0ull, 0ull};
     MSCD_CUDA(cudaMallocAsync((void **)&ps, sizeof(PrepState), st));
     int rc = MSCD_OK;
     PrepState h{};
-    i64 nnz = 0;
     do {
+        // one wait: a kernel that an earlier one's findings make pointless returns at once
         if ((rc = cuda_status(cudaMemcpyAsync(ps, &init, sizeof(init), cudaMemcpyHostToDevice, st)))) break;
-        check_row_ptr<<<(unsigned)((n + 1 + 255) / 256), 256, 0, st>>>(rp, n, ps); note_launch();
-        if ((rc = cuda_status(cudaMemcpyAsync(&h, ps, sizeof(h), cudaMemcpyDeviceToHost, st)))) break;
-        if ((rc = cuda_status(cudaStreamSynchronize(st)))) break;
-        if (h.mask) { rc = MSCD_EINVAL; break; }
-        if ((rc = cuda_status(cudaMemcpyAsync(&nnz, rp + n, sizeof(i64), cudaMemcpyDeviceToHost, st)))) break;
-        if ((rc = cuda_status(cudaStreamSynchronize(st)))) break;
-        const unsigned row_blocks = (unsigned)std::max<i64>(1, std::min<i64>((n + 7) / 8, 152 * 64));
-        if (n > 0) { check_entries<<<row_blocks, 256, 0, st>>>(rp, col, w, n, ps); note_launch(); }
-        if ((rc = cuda_status(cudaMemcpyAsync(&h, ps, sizeof(h), cudaMemcpyDeviceToHost, st)))) break;
-        if ((rc = cuda_status(cudaStreamSynchronize(st)))) break;
-        if ((rc = first_category(h.mask))) break;
-        int ue = 0;
-        if (w && nnz > 0) {
-            ue = h.min_lowbit;
-            if ((rc = cuda_status(cudaMalloc((void **)wfx_out, (size_t)nnz * sizeof(i64))))) break;
-            fixed_weights<<<(unsigned)std::min<i64>((nnz + 255) / 256, 152 * 32), 256, 0, st>>>(w, nnz, ue,
-                                                                                             *wfx_out, ps); note_launch();
+        check_row_ptr<<<(unsigned)((n + 1 + 255) / 256), 256, 0, st>>>(rp, n, nnz, ps); note_launch();
+        if (n > 0) {
+            const unsigned row_blocks = (unsigned)std::min<i64>((n + 7) / 8, 152 * 8);
+            check_entries<<<row_blocks, 256, 0, st>>>(rp, col, w, n, ps); note_launch();
+            if (w) {
+                weighted_degrees<<<(unsigned)std::min<i64>((n + 15) / 16, 152 * 8), 256, 0, st>>>(rp, w, n, wfx, k,
+                                                                                                  logk, ps);
+            } else {
+                degrees<<<(unsigned)std::min<i64>((n + 255) / 256, 152 * 8), 256, 0, st>>>(rp, n, k, logk, ps);
+            }
+            note_launch();
         }
-        if ((rc = cuda_status(cudaMalloc((void **)k_out, (size_t)std::max<i64>(n, 1) * sizeof(i64))))) break;
-        if ((rc = cuda_status(cudaMalloc((void **)logk_out, (size_t)std::max<i64>(n, 1) * sizeof(float))))) break;
-        if (n > 0) { degrees<<<row_blocks, 256, 0, st>>>(rp, *wfx_out, n, *k_out, *logk_out, ps); note_launch(); }
         if ((rc = cuda_status(cudaMemcpyAsync(&h, ps, sizeof(h), cudaMemcpyDeviceToHost, st)))) break;
         if ((rc = cuda_status(cudaStreamSynchronize(st)))) break;
+        if ((rc = cuda_status(cudaGetLastError()))) break;
+        // CAT_RANGE comes after the symmetry found by the count
+        if (!(h.mask & ~(u32)CAT_RANGE) && h.below) h.mask |= CAT_NOTSYM;
         if ((rc = first_category(h.mask))) break;
         if (h.total_d >= 0x1p63 || h.total >= (1ull << 62)) { rc = MSCD_ERANGE; break; }
         g->n = n;
         g->nnz = nnz;
         g->rp = rp;
         g->col = col;
-        g->wfx = *wfx_out;
-        g->k = *k_out;
-        g->logk = *logk_out;
-        g->unit_exp = ue;
+        g->wfx = w && nnz > 0 ? wfx : nullptr;
+        g->k = k;
+        g->logk = logk;
+        g->unit_exp = w && nnz > 0 ? h.min_lowbit : 0;
         g->volume = (i64)h.total;
         g->kmax = (i64)h.kmax;
     } while (0);
     cudaFreeAsync(ps, st);
-    if (rc != MSCD_OK) {
-        cudaStreamSynchronize(st);
-        if (*wfx_out) cudaFree(*wfx_out);
-        if (*k_out) cudaFree(*k_out);
-        if (*logk_out) cudaFree(*logk_out);
-        *wfx_out = nullptr;
-        *k_out = nullptr;
-        *logk_out = nullptr;
-    }
+    if (rc != MSCD_OK) cudaStreamSynchronize(st);
     return rc;
 }
