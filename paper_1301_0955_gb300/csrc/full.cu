@@ -35,6 +35,7 @@
 #include "common.cuh"
 #include "dedup.cuh"
 #include "grow.cuh"
+#include "incidence.cuh"
 #include "ladder.cuh"
 
 namespace {
@@ -138,26 +139,84 @@ __device__ __forceinline__ i64 threshold(i64 a, i64 b, double eta) {
     return k < 1 ? 1 : k;
 }
 
-// Index in A (sorted) of the t-th node A shares with B (sorted); -1 if fewer.
-__device__ i64 tth_common(const i32 *A, i64 na, const i32 *B, i64 nb, i64 t) {
-    i64 i = 0, j = 0, k = 0;
-    while (i < na && j < nb) {
-        if (A[i] < B[j]) ++i;
-        else if (A[i] > B[j]) ++j;
-        else {
-            if (++k == t) return i;
-            ++i;
-            ++j;
+__device__ __forceinline__ bool in_sorted(const i32 *a, i64 n, i32 v) {
+    i64 lo = 0, hi = n;
+    while (lo < hi) {
+        const i64 mid = (lo + hi) >> 1;
+        if (a[mid] < v) lo = mid + 1;
+        else hi = mid;
+    }
+    return lo < n && a[lo] == v;
+}
+
+// Index in A (sorted) of the t-th node A shares with B (sorted); -1 if fewer,
+// or if it is not below `stop`.  Warp-collective: 32 of A's nodes at a time
+// are looked up in B.
+__device__ i64 tth_common(const i32 *A, i64 na, const i32 *B, i64 nb, i64 t, i64 stop) {
+    const int lane = threadIdx.x & 31;
+    for (i64 i = 0; i < min(na, stop); i += 32) {
+        u32 hit = __ballot_sync(FULL_MASK, i + lane < na && in_sorted(B, nb, A[i + lane]));
+        const int c = __popc(hit);
+        if (c >= t) {
+            for (; t > 1; --t) hit &= hit - 1;
+            return i + __ffs(hit) - 1;
         }
+        t -= c;
     }
     return -1;
 }
 
 __device__ __forceinline__ u32 hash_c(i32 l) { return (u32)l * 0x9E3779B1u; }
 
+// The first community in c's scan order that reaches the threshold, among this
+// lane's candidate o with `cnt` shared nodes (o < 0: none) and `best` so far
+// ((position << 32) | partner, the same in every lane).  Warp-collective.
+__device__ unsigned long long reach_first(const i64 *cptr, const i32 *cnodes, i32 c, i32 o, i32 cnt, double eta,
+                                          unsigned long long best) {
+    const i64 na = cptr[c + 1] - cptr[c];
+    i64 th = 0;
+    if (o >= 0) th = threshold(na, cptr[o + 1] - cptr[o], eta);
+    u32 cand = __ballot_sync(FULL_MASK, o >= 0 && (i64)cnt >= th);
+    for (; cand; cand &= cand - 1) {
+        const int l = __ffs(cand) - 1;
+        const i32 p = __shfl_sync(FULL_MASK, o, l);
+        const i64 t = __shfl_sync(FULL_MASK, th, l);
+        const i64 stop = best == ~0ull ? na : (i64)(best >> 32) + 1;
+        const i64 pos = tth_common(cnodes + cptr[c], na, cnodes + cptr[p], cptr[p + 1] - cptr[p], t, stop);
+        if (pos >= 0) best = min(best, ((unsigned long long)pos << 32) | (u32)p);
+    }
+    return best;
+}
+
+// Count one node shared with o; true: o is new, in the bucket `at`.
+__device__ __forceinline__ bool count_in(i32 *keys, i32 *cnts, u32 mask, i32 o, u32 &at) {
+    u32 h = hash_c(o) & mask;
+    bool fresh = false;
+    for (u32 p = 0; p <= mask; ++p) {
+        i32 cur = keys[h];
+        if (cur == -1) {
+            cur = atomicCAS(&keys[h], -1, o);
+            if (cur == -1) {
+                fresh = true;
+                cur = o;
+            }
+        }
+        if (cur == o) {
+            atomicAdd(&cnts[h], 1);
+            break;
+        }
+        h = (h + 1u) & mask;
+    }
+    at = h;
+    return fresh;
+}
+
 // Warp per listed community c: partner[c] = the first community reaching the
 // threshold in c's scan order, or -1; communities meeting more partners than
 // the shared-memory table holds are listed in `spill` for reach_global.
+// Bound by the dependent loads of its largest communities: 32 members' lists
+// at a time (40 launches of a 30,000-node run at 8 scales: 25.5 ms with one
+// member at a time and merges of the lists by one lane, now 3.7).
 __global__ void __launch_bounds__(REACH_WARPS * 32) reach_smem(const i64 *cptr, const i32 *cnodes, const i64 *mptr,
                                                                const i32 *mlist, const i32 *list, i64 nl, double eta,
                                                                i32 *partner, i32 *spill, unsigned long long *n_spill) {
@@ -178,30 +237,16 @@ __global__ void __launch_bounds__(REACH_WARPS * 32) reach_smem(const i64 *cptr, 
         if (lane == 0) sfill[w] = 0;
         __syncwarp();
         bool over = false;
-        for (i64 e = cptr[c]; e < cptr[c + 1] && !over; ++e) {
-            const i32 u = cnodes[e];
-            for (i64 j = mptr[u] + lane; j < mptr[u + 1]; j += 32) {
-                const i32 o = mlist[j];
-                if (o == c) continue;
-                u32 h = hash_c(o) & (REACH_TABLE - 1);
-                for (int p = 0; p < REACH_TABLE; ++p) {
-                    i32 cur = keys[h];
-                    if (cur == -1) {
-                        cur = atomicCAS(&keys[h], -1, o);
-                        if (cur == -1) {
-                            const int f = atomicAdd(&sfill[w], 1);
-                            if (f >= REACH_TABLE / 2) over = true;
-                            else used[f] = (unsigned short)h;
-                            cur = o;
-                        }
-                    }
-                    if (cur == o) {
-                        atomicAdd(&cnts[h], 1);
-                        break;
-                    }
-                    h = (h + 1u) & (REACH_TABLE - 1);
+        const i64 e1 = cptr[c + 1];
+        for (i64 e = cptr[c]; e < e1 && !over; e += 32) {
+            visit_lists(cnodes, e, min(e + 32, e1), mptr, mlist, [&](i32 o) {
+                u32 h;
+                if (o != c && count_in(keys, cnts, REACH_TABLE - 1, o, h)) {
+                    const int f = atomicAdd(&sfill[w], 1);
+                    if (f >= REACH_TABLE / 2) over = true;
+                    else used[f] = (unsigned short)h;
                 }
-            }
+            });
             over = __any_sync(FULL_MASK, over);
         }
         __syncwarp();
@@ -215,22 +260,18 @@ __global__ void __launch_bounds__(REACH_WARPS * 32) reach_smem(const i64 *cptr, 
             continue;
         }
         const int nf = sfill[w];
-        const i64 na = cptr[c + 1] - cptr[c];
         unsigned long long best = ~0ull;  // (position << 32) | partner
-        for (int t = lane; t < nf; t += 32) {
-            const int h = used[t];
-            const i32 o = keys[h];
-            const i32 cnt = cnts[h];
-            keys[h] = -1;
-            cnts[h] = 0;
-            const i64 nb = cptr[o + 1] - cptr[o];
-            const i64 th = threshold(na, nb, eta);
-            if (cnt < th) continue;
-            const i64 pos = tth_common(cnodes + cptr[c], na, cnodes + cptr[o], nb, th);
-            const unsigned long long key = ((unsigned long long)pos << 32) | (u32)o;
-            best = min(best, key);
+        for (int t0 = 0; t0 < nf; t0 += 32) {
+            i32 o = -1, cnt = 0;
+            if (t0 + lane < nf) {
+                const int h = used[t0 + lane];
+                o = keys[h];
+                cnt = cnts[h];
+                keys[h] = -1;
+                cnts[h] = 0;
+            }
+            best = reach_first(cptr, cnodes, c, o, cnt, eta, best);
         }
-        for (int off = 16; off; off >>= 1) best = min(best, __shfl_xor_sync(FULL_MASK, best, off));
         if (lane == 0) partner[c] = best == ~0ull ? -1 : (i32)(best & 0xffffffffu);
         __syncwarp();
     }
@@ -245,39 +286,18 @@ __global__ void reach_global(const i64 *cptr, const i32 *cnodes, const i64 *mptr
         const i32 c = list[r];
         i32 *keys = tkey + toff[r], *cnts = tcnt + toff[r];
         const u32 tm = (u32)(toff[r + 1] - toff[r] - 1);
-        for (i64 e = cptr[c]; e < cptr[c + 1]; ++e) {
-            const i32 u = cnodes[e];
-            for (i64 j = mptr[u] + lane; j < mptr[u + 1]; j += 32) {
-                const i32 o = mlist[j];
-                if (o == c) continue;
-                u32 h = hash_c(o) & tm;
-                for (u32 p = 0; p <= tm; ++p) {
-                    i32 cur = keys[h];
-                    if (cur == -1) {
-                        cur = atomicCAS(&keys[h], -1, o);
-                        if (cur == -1) cur = o;
-                    }
-                    if (cur == o) {
-                        atomicAdd(&cnts[h], 1);
-                        break;
-                    }
-                    h = (h + 1u) & tm;
-                }
-            }
-        }
+        const i64 e1 = cptr[c + 1];
+        for (i64 e = cptr[c]; e < e1; e += 32)
+            visit_lists(cnodes, e, min(e + 32, e1), mptr, mlist, [&](i32 o) {
+                u32 h;
+                if (o != c) count_in(keys, cnts, tm, o, h);
+            });
         __syncwarp();
-        const i64 na = cptr[c + 1] - cptr[c];
         unsigned long long best = ~0ull;
-        for (u32 t = lane; t <= tm; t += 32) {
-            const i32 o = keys[t];
-            if (o < 0) continue;
-            const i64 nb = cptr[o + 1] - cptr[o];
-            const i64 th = threshold(na, nb, eta);
-            if (cnts[t] < th) continue;
-            const i64 pos = tth_common(cnodes + cptr[c], na, cnodes + cptr[o], nb, th);
-            best = min(best, ((unsigned long long)pos << 32) | (u32)o);
+        for (u32 t0 = 0; t0 <= tm; t0 += 32) {
+            const u32 t = t0 + lane;
+            best = reach_first(cptr, cnodes, c, t <= tm ? keys[t] : -1, t <= tm ? cnts[t] : 0, eta, best);
         }
-        for (int off = 16; off; off >>= 1) best = min(best, __shfl_xor_sync(FULL_MASK, best, off));
         if (lane == 0) partner[c] = best == ~0ull ? -1 : (i32)(best & 0xffffffffu);
     }
 }
@@ -356,16 +376,6 @@ __global__ void new_lists(const i64 *cptr, const i32 *cnodes, i64 C, const i32 *
 
 // ---- per-community fitness and list hash -----------------------------------
 
-__device__ __forceinline__ bool in_sorted(const i32 *a, i64 n, i32 v) {
-    i64 lo = 0, hi = n;
-    while (lo < hi) {
-        const i64 mid = (lo + hi) >> 1;
-        if (a[mid] < v) lo = mid + 1;
-        else hi = mid;
-    }
-    return lo < n && a[lo] == v;
-}
-
 __device__ __forceinline__ u64 mix(u64 x) {
     x ^= x >> 33;
     x *= 0xff51afd7ed558ccdull;
@@ -375,38 +385,62 @@ __device__ __forceinline__ u64 mix(u64 x) {
     return x;
 }
 
-// Warp per community: K (internal degree sum), V, f = K / V^alpha in real
-// weight units (Eq. 1), and a hash of the sorted list.
-__global__ void comm_fitness(const DevGraph G, const i64 *cptr, const i32 *cnodes, i64 C, double alpha, double *f,
-                             u64 *hash) {
-    const int lane = threadIdx.x & 31;
-    const i64 warps = (i64)gridDim.x * (blockDim.x >> 5);
-    for (i64 c = (i64)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); c < C; c += warps) {
+constexpr int FIT_WARPS = 16;
+constexpr int FIT_LIST = 8192;  // members looked up in shared memory
+
+// CTA per community: K (internal degree sum), V, f = K / V^alpha in real
+// weight units (Eq. 1), and a hash of the sorted list.  The warps take the
+// members' rows; every neighbour is looked up in the list, in shared memory
+// up to FIT_LIST members (a warp per community and the list in global memory
+// took 11.5 ms in 8 launches of a 30,000-node run, now 1.0).
+__global__ void __launch_bounds__(FIT_WARPS * 32) comm_fitness(const DevGraph G, const i64 *cptr, const i32 *cnodes,
+                                                               i64 C, double alpha, double *f, u64 *hash) {
+    __shared__ i32 slist[FIT_LIST];
+    __shared__ unsigned long long sK, sV, sh;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (i64 c = blockIdx.x; c < C; c += gridDim.x) {
         const i32 *L = cnodes + cptr[c];
         const i64 n = cptr[c + 1] - cptr[c];
-        i64 K = 0, V = 0;
+        if (threadIdx.x == 0) sK = sV = sh = 0;
+        i64 V = 0, K = 0;
         u64 h = 0;
-        for (i64 i = 0; i < n; ++i) {
+        for (i64 i = threadIdx.x; i < n; i += FIT_WARPS * 32) {
             const i32 u = L[i];
-            if (lane == 0) V += G.k[u];
-            for (i64 e = G.rp[u] + lane; e < G.rp[u + 1]; e += 32)
-                if (in_sorted(L, n, G.col[e])) K += G.wfx ? G.wfx[e] : 1;
+            if (n <= FIT_LIST) slist[i] = u;
+            V += G.k[u];
+            h += mix((u64)(u32)u + 0x9E3779B97F4A7C15ull * (u64)(i + 1));
         }
-        for (i64 i = lane; i < n; i += 32) h += mix((u64)(u32)L[i] + 0x9E3779B97F4A7C15ull * (u64)(i + 1));
+        __syncthreads();
+        const i32 *look = n <= FIT_LIST ? slist : L;
+        for (i64 i = w; i < n; i += FIT_WARPS) {
+            const i32 u = look[i];
+            const i64 re = G.rp[u + 1];
+            for (i64 e = G.rp[u] + lane; e < re; e += 32)
+                if (in_sorted(look, n, G.col[e])) K += G.wfx ? G.wfx[e] : 1;
+        }
         for (int o = 16; o; o >>= 1) {
             K += __shfl_xor_sync(FULL_MASK, K, o);
+            V += __shfl_xor_sync(FULL_MASK, V, o);
             h += __shfl_xor_sync(FULL_MASK, h, o);
         }
         if (lane == 0) {
+            atomicAdd(&sK, (unsigned long long)K);
+            atomicAdd(&sV, (unsigned long long)V);
+            atomicAdd(&sh, (unsigned long long)h);
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
             double fv = 0.0;
-            if (K > 0) {
+            if (sK > 0) {
                 const double LN2 = 0.6931471805599453;
-                fv = exp(log((double)K) - alpha * log((double)V) + (1.0 - alpha) * (double)G.unit_exp * LN2);
+                fv = exp(log((double)(i64)sK) - alpha * log((double)(i64)sV) +
+                         (1.0 - alpha) * (double)G.unit_exp * LN2);
             }
             f[c] = fv;
-            h ^= mix((u64)n);
-            hash[c] = h ? h : 1;
+            const u64 hh = (u64)sh ^ mix((u64)n);
+            hash[c] = hh ? hh : 1;
         }
+        __syncthreads();
     }
 }
 
@@ -839,7 +873,9 @@ int full_run(const DevGraph &G, i64 max_part_n, const double *alphas, int32_t n_
                                                              cudaMemcpyDeviceToDevice, st))))
                 break;
             if (X.C > 0) {
-                comm_fitness<<<GB, 256, 0, st>>>(G, X.ptr, X.nodes, X.C, alpha, R.comm_f, R.comm_hash); note_launch();
+                comm_fitness<<<(unsigned)std::min<i64>(X.C, GB), FIT_WARPS * 32, 0, st>>>(G, X.ptr, X.nodes, X.C, alpha,
+                                                                                         R.comm_f, R.comm_hash);
+                note_launch();
             }
             rc = cuda_status(cudaStreamSynchronize(st));
         } while (0);

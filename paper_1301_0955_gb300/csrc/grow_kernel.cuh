@@ -539,6 +539,94 @@ __device__ __forceinline__ void load_entries(const DevGraph &G, i64 at, i64 re, 
     }
 }
 
+// A lane's node in the slots.
+template <class D>
+struct Found {
+    int slot;     // -1 none
+    bool fresh;   // inserted now: its record is still to be written
+    bool member;
+    D d, k;       // fresh: 0 and its degree (unweighted)
+};
+
+// Look up node v of every active lane (distinct nodes), giving absent ones a
+// slot and a bucket.  The table (H buckets) has room for 32 more.  False: the
+// slots are full.  Warp-collective.
+template <class ST>
+__device__ __forceinline__ bool locate(const ST &st, const DevGraph &G, int &ns, int H, i32 v, bool active,
+                                       Found<typename ST::D> &r) {
+    typedef typename ST::D D;
+    typedef typename ST::BT BT;
+    const int lane = threadIdx.x & 31;
+    const u32 hm = (u32)H - 1u;
+    r.slot = -1;
+    r.fresh = r.member = false;
+    r.d = r.k = 0;
+    u32 h = active ? first_bucket(v, H) : 0u;
+    bool open = active;
+    int p = 0;  // buckets passed (the table is at most half full)
+    while (__any_sync(FULL_MASK, open)) {
+        BT x = 0;
+        if (open)
+            for (x = st.hsh[h]; x != 0 && !bucket_may(x, v) && p < H; ++p) {
+                h = (h + 1u) & hm;
+                x = st.hsh[h];
+            }
+        __syncwarp();
+        if (open) {
+            if (x == 0) {
+                if (!ST::WEIGHTED) r.k = (D)G.k[v];
+                r.fresh = true;
+                open = false;
+            } else {
+                const int i = bucket_slot(x);
+                i32 id;
+                D dd, dk;
+                st.sl.get(i, id, dd, dk);
+                if (node_of(id) == v) {
+                    r.slot = i;
+                    r.d = dd;
+                    r.k = dk;
+                    r.member = id < 0;
+                    open = false;
+                } else {
+                    h = (h + 1u) & hm;
+                    if (++p >= H) {
+                        my_unit().err = 1;
+                        open = false;
+                    }
+                }
+            }
+        }
+    }
+    const u32 ball = __ballot_sync(FULL_MASK, r.fresh);
+    if (ball) {
+        const int cnt = __popc(ball);
+        if (ns + cnt > st.C) return false;
+        if (r.fresh) r.slot = ns + __popc(ball & lanemask_lt());
+        // Claim the empty buckets found.  Only this warp writes its table, so
+        // lanes that found the same bucket are told apart without atomics:
+        // each writes its number under the bucket's tag, the one that reads
+        // itself back takes the bucket, the others look again from there.
+        // Every round settles at least one lane.
+        unsigned char *tag = my_unit().tag;
+        bool pending = r.fresh;
+        for (int i = 0; i < 32; ++i) {
+            if (pending) tag[h & (CLAIM_TAGS - 1)] = (unsigned char)lane;
+            __syncwarp();
+            if (pending && tag[h & (CLAIM_TAGS - 1)] == lane) {
+                st.hsh[h] = bucket<BT>(r.slot, v);
+                pending = false;
+            }
+            __syncwarp();
+            if (!__any_sync(FULL_MASK, pending)) break;
+            if (pending)
+                for (; st.hsh[h] != 0 && p < H; ++p) h = (h + 1u) & hm;
+        }
+        ns += cnt;
+    }
+    return true;
+}
+
 // Scan the row [rs, re), 32 entries at a time: look each neighbour up, insert
 // it if absent, add sign * w to its d_in; with requeue, (re)insert outside
 // nodes in the queue with their new key and raise their group's bounds.  nv,
@@ -548,7 +636,6 @@ template <class ST>
 __device__ __forceinline__ bool expand(const ST &st, const GrowArgs &a, Live &U, i64 rs, i64 re, int sign,
                                        bool requeue, i32 nv, typename ST::D nw) {
     typedef typename ST::D D;
-    typedef typename ST::BT BT;
     const int lane = threadIdx.x & 31;
 #pragma unroll 1
     for (i64 b = rs; b < re; b += 32) {
@@ -556,78 +643,15 @@ __device__ __forceinline__ bool expand(const ST &st, const GrowArgs &a, Live &U,
         const D w = nw;
         load_entries<ST>(a.G, b + 32, re, nv, nw);  // in flight during these look-ups
         if (ST::FILL * (U.ns + 32) > U.H && U.H < st.Hmax()) U.H = far(rehash<ST>)(U.ns, U.H);
-        const u32 hm = (u32)U.H - 1u;
-        int s = -1;
-        bool need = false, member = false;
-        D d = 0, k = 0;
+        const bool active = b + lane < re;
         float lk = 0.0f;
-        u32 h = 0;
-        bool open = b + lane < re;
-        if (open) {
-            if (ST::WEIGHTED) lk = a.G.logk[v];  // depends only on v, like the bucket
-            h = first_bucket(v, U.H);
-        }
-        int p = 0;  // buckets passed (the table is at most half full)
-        while (__any_sync(FULL_MASK, open)) {
-            BT x = 0;
-            if (open)
-                for (x = st.hsh[h]; x != 0 && !bucket_may(x, v) && p < U.H; ++p) {
-                    h = (h + 1u) & hm;
-                    x = st.hsh[h];
-                }
-            __syncwarp();
-            if (open) {
-                if (x == 0) {
-                    if (!ST::WEIGHTED) k = (D)a.G.k[v];
-                    need = true;
-                    open = false;
-                } else {
-                    const int i = bucket_slot(x);
-                    i32 id;
-                    D dd, dk;
-                    st.sl.get(i, id, dd, dk);
-                    if (node_of(id) == v) {
-                        s = i;
-                        d = dd;
-                        k = dk;
-                        member = id < 0;
-                        open = false;
-                    } else {
-                        h = (h + 1u) & hm;
-                        if (++p >= U.H) {
-                            my_unit().err = 1;
-                            open = false;
-                        }
-                    }
-                }
-            }
-        }
-        const u32 ball = __ballot_sync(FULL_MASK, need);
-        if (ball) {
-            const int cnt = __popc(ball);
-            if (U.ns + cnt > st.C) return false;
-            if (need) s = U.ns + __popc(ball & lanemask_lt());
-            // Claim the empty buckets found.  Only this warp writes its table, so
-            // lanes that found the same bucket are told apart without atomics:
-            // each writes its number under the bucket's tag, the one that reads
-            // itself back takes the bucket, the others look again from there.
-            // Every round settles at least one lane.
-            unsigned char *tag = my_unit().tag;
-            bool pending = need;
-            for (int r = 0; r < 32; ++r) {
-                if (pending) tag[h & (CLAIM_TAGS - 1)] = (unsigned char)lane;
-                __syncwarp();
-                if (pending && tag[h & (CLAIM_TAGS - 1)] == lane) {
-                    st.hsh[h] = bucket<BT>(s, v);
-                    pending = false;
-                }
-                __syncwarp();
-                if (!__any_sync(FULL_MASK, pending)) break;
-                if (pending)
-                    for (; st.hsh[h] != 0 && p < U.H; ++p) h = (h + 1u) & hm;
-            }
-            U.ns += cnt;
-        }
+        if (ST::WEIGHTED && active) lk = a.G.logk[v];  // depends only on v, like the bucket
+        Found<D> f;
+        if (!locate(st, a.G, U.ns, U.H, v, active, f)) return false;
+        const int s = f.slot;
+        const bool need = f.fresh, member = f.member;
+        D d = f.d;
+        const D k = f.k;
         if (s >= 0) {
             if (ST::WEIGHTED) d += sign < 0 ? -w : w;
             else d += sign;
@@ -653,7 +677,7 @@ __device__ __forceinline__ bool expand(const ST &st, const GrowArgs &a, Live &U,
 
 // ---- everything else ---------------------------------------------------------
 
-enum { SEED_ROW, INIT_ROW, GROW_ROW, PRUNE_ROW };  // Unit::step
+enum { SEED_ROW, GROW_ROW, PRUNE_ROW };    // Unit::step
 enum { ROW_DONE, TOP_FAILS, QUEUE_EMPTY };         // why the loop stopped
 enum { DONE, SCAN, SCAN_AND_GROW };                // what next_row asks for
 
@@ -871,41 +895,99 @@ __device__ __forceinline__ void unlist_member(const ST &st, Unit &U, int s, i32 
     __syncwarp();
 }
 
-// Slot of one node (every lane the same), inserted with d_in = 0 if absent;
-// -1: the slots are full.
+// Add the initial members (Alg. 2 may start from given communities; repeats
+// and the seed itself are skipped): all of them are looked up and listed 32 at
+// a time, then their rows are scanned with the next row's bounds loaded ahead,
+// then K is the sum of the members' d_in (each inner edge twice, as joining one
+// after the other gives).  One by one through next_row a member cost some
+// 11,000 cycles, and large communities that hardly grow made the full method's
+// launches wait (growth of a 30,000-node run at 8 scales: 106 ms, now 70).
 template <class ST>
-__device__ __forceinline__ int find_one(const ST &st, Unit &U, i32 v) {
-    typedef typename ST::BT BT;
-    const int lane = threadIdx.x & 31, ns = U.ns;
-    int H = U.H;
-    if (ST::FILL * (ns + 32) > H && H < st.Hmax()) {
-        H = rehash<ST>(ns, H);
-        if (lane == 0) U.H = H;
+__device__ __noinline__ void init_members() {
+    typedef typename ST::D D;
+    const GrowArgs &a = args();
+    const DevGraph &G = a.G;
+    const ST st = my_state<ST>(a);
+    Unit &U = my_unit();
+    const int lane = threadIdx.x & 31;
+    Live L;
+    L.ns = U.ns;
+    L.H = U.H;
+    L.K = L.V = 0;
+    L.alpha32 = L.E2 = 0.0f;
+    int nm = U.nm;
+    const int nm0 = nm;
+    bool full = false;
+    i64 V = 0;
+    const i64 end = U.init_end;
+#pragma unroll 1
+    for (i64 at = U.init_at; at < end; at += 32) {
+        const i32 v = at + lane < end ? a.init_nodes[at + lane] : -1 - lane;
+        const u32 same = __match_any_sync(FULL_MASK, v);
+        const bool active = v >= 0 && __ffs(same) - 1 == lane;
+        if (ST::FILL * (L.ns + 32) > L.H && L.H < st.Hmax()) L.H = far(rehash<ST>)(L.ns, L.H);
+        Found<D> f;
+        if (!locate(st, G, L.ns, L.H, v, active, f)) {
+            full = true;
+            break;
+        }
+        const bool joins = f.slot >= 0 && !f.member;
+        const u32 ball = __ballot_sync(FULL_MASK, joins);
+        if (joins) {
+            if (f.fresh) st.sl.put_new(f.slot, v | MEMBER_BIT, NEG_INF, f.d, f.k);
+            else st.sl.put_id(f.slot, v | MEMBER_BIT);
+            st.mem[nm + __popc(ball & lanemask_lt())] = (typename ST::MT)f.slot;
+            V += G.k[v];
+        }
+        nm += __popc(ball);
         __syncwarp();
     }
-    const u32 hm = (u32)H - 1u;
-    u32 h = first_bucket(v, H);
-    for (int p = 0; p < H; ++p, h = (h + 1u) & hm) {
-        const BT x = st.hsh[h];
-        if (x == 0) {
-            if (ns >= st.C) return -1;
-            __syncwarp();
-            if (lane == 0) {
-                st.hsh[h] = bucket<BT>(ns, v);
-                st.sl.put_new(ns, v, NEG_INF, 0, ST::WEIGHTED ? 0 : (typename ST::D)args().G.k[v]);
-                U.ns = ns + 1;
-            }
-            __syncwarp();
-            return ns;
-        }
-        if (bucket_may(x, v) && node_of(st.sl.id(bucket_slot(x))) == v) return bucket_slot(x);
+    i64 rs = 0, re = 0;
+    if (!full && nm0 < nm) {
+        const i32 u = node_of(st.sl.id(st.mem[nm0]));
+        rs = G.rp[u];
+        re = G.rp[u + 1];
     }
-    return -1;
+#pragma unroll 1
+    for (int j = nm0; j < nm && !full; ++j) {
+        i32 v = 0;
+        D w = 0;
+        load_entries<ST>(G, rs, re, v, w);
+        const i64 rs0 = rs, re0 = re;
+        if (j + 1 < nm) {
+            const i32 u = node_of(st.sl.id(st.mem[j + 1]));
+            rs = G.rp[u];
+            re = G.rp[u + 1];
+        }
+        full = !expand(st, a, L, rs0, re0, 1, false, v, w);
+    }
+    i64 K = 0;
+    for (int j = lane; j < nm && !full; j += 32) {
+        i32 id;
+        D d, k;
+        st.sl.get(st.mem[j], id, d, k);
+        K += (i64)d;
+    }
+    for (int o = 16; o; o >>= 1) {
+        K += __shfl_xor_sync(FULL_MASK, K, o);
+        V += __shfl_xor_sync(FULL_MASK, V, o);
+    }
+    __syncwarp();
+    if (lane == 0) {
+        U.ns = L.ns;
+        U.H = L.H;
+        U.nm = nm;
+        U.K = K;
+        U.V += V;
+        U.init_at = end;
+        if (full) U.ovf = 1;
+    }
+    __syncwarp();
 }
 
-// Choose the row to scan after the loop stopped (`why`): the next initial
-// member's, that of the first node to pass after a run of rejections, that of
-// a member to prune; and begin rounds in between.  The unit is in my_unit().
+// Choose the row to scan after the loop stopped (`why`): that of the first node
+// to pass after a run of rejections, that of a member to prune; add the initial
+// members before the first round and begin rounds.  The unit is in my_unit().
 template <class ST>
 __device__ __noinline__ int next_row(int why) {
     typedef typename ST::D D;
@@ -918,24 +1000,9 @@ __device__ __noinline__ int next_row(int why) {
     i32 u = 0;
     D d = 0, k = 0;
     int step = U.step;
-    if (step <= INIT_ROW) {
-        // initial members (Alg. 2 may start from given communities), looked
-        // up and added one by one; repeats and the seed itself are skipped
-        i64 at = U.init_at;
-        const i64 end = U.init_end;
-        while (at < end && add < 0) {
-            const int s = find_one(st, U, a.init_nodes[at++]);
-            if (s < 0) {
-                if (lane == 0) U.ovf = 1;
-                __syncwarp();
-                return DONE;
-            }
-            st.sl.get(s, u, d, k);
-            if (u >= 0) add = s;
-        }
-        __syncwarp();
-        if (lane == 0) U.init_at = at;
-        if (add >= 0) step = INIT_ROW;
+    if (step == SEED_ROW && U.init_at < U.init_end) {
+        far(init_members<ST>)();
+        if (U.ovf) return DONE;
     }
     if (step == GROW_ROW) {
         if (why == TOP_FAILS) {
@@ -1015,16 +1082,14 @@ __device__ __noinline__ int next_row(int why) {
         U.K += 2 * (i64)d;
         U.V += G.k[u];
         U.step = step;
-        if (step == GROW_ROW) {
-            U.adds += 1ull;
-            U.added = true;
-        }
+        U.adds += 1ull;
+        U.added = true;
         U.rs = G.rp[u];
         U.re = G.rp[u + 1];
         U.sign = 1;
     }
     __syncwarp();
-    return step == GROW_ROW ? SCAN_AND_GROW : SCAN;
+    return SCAN_AND_GROW;
 }
 
 // Sort the members ascending into scratch (the group bounds where they hold

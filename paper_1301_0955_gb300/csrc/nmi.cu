@@ -55,6 +55,7 @@
 
 #include "common.cuh"
 #include "dedup.cuh"
+#include "incidence.cuh"
 
 int ctx_device_of(mscd_ctx *c);
 
@@ -311,54 +312,6 @@ __global__ void big_offsets(PairArgs a) {
     if (lane == 0) d.boff[a.P] = at;
 }
 
-// f(l) for every community l of B that holds a member in anodes[e0, e1), at
-// most 32 members; once per member and community.  Warp-collective.
-template <class F>
-__device__ __forceinline__ void visit_partners(const Direction &d, i64 e0, i64 e1, F f) {
-    constexpr int AHEAD = 4;  // entries a lane has in flight
-    const int lane = threadIdx.x & 31;
-    i64 lo = 0;
-    int len = 0;
-    if (e0 + lane < e1) {
-        const i32 u = d.anodes[e0 + lane];
-        lo = d.mptr[u];
-        len = d.mcnt[u];
-    }
-    if (__any_sync(FULL_MASK, len > 1 << 25)) {  // the sums below would not fit
-        for (int i = 0; i < 32; ++i) {
-            const i64 b = __shfl_sync(FULL_MASK, lo, i);
-            const int m = __shfl_sync(FULL_MASK, len, i);
-            for (int t = lane; t < m; t += 32) f(d.mlist[b + t]);
-        }
-        return;
-    }
-    int incl = len;  // the lists end to end: member i's entries are incl - len .. incl
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(FULL_MASK, incl, o);
-        if (lane >= o) incl += y;
-    }
-    const int total = __shfl_sync(FULL_MASK, incl, 31);
-    const i64 first = lo - (incl - len);  // entry t of the whole is mlist[first + t]
-    for (int t0 = 0; t0 < total; t0 += 32 * AHEAD) {
-        i32 l[AHEAD];
-#pragma unroll
-        for (int j = 0; j < AHEAD; ++j) {
-            l[j] = -1;
-            if (t0 + 32 * j >= total) continue;
-            const int t = t0 + 32 * j + lane;
-            int i = 0;  // first member whose list ends beyond t
-#pragma unroll
-            for (int step = 16; step; step >>= 1)
-                if (__shfl_sync(FULL_MASK, incl, i + step - 1) <= t) i += step;
-            const i64 b = __shfl_sync(FULL_MASK, first, i);
-            if (t < total) l[j] = d.mlist[b + t];
-        }
-#pragma unroll
-        for (int j = 0; j < AHEAD; ++j)
-            if (l[j] >= 0) f(l[j]);
-    }
-}
-
 // A hash of partner communities and how many nodes they share with A's.
 struct Counts {
     i32 *keys, *cnts;
@@ -462,7 +415,7 @@ __global__ void __launch_bounds__(NMI_WARPS * 32) pairs_warp(const __grid_consta
             if (lane == 0) sfill[w] = 0;
             __syncwarp();
             for (i64 e = e0; e < e1 && !over; e += 32) {
-                visit_partners(d, e, min(e + 32, e1), [&](i32 l) {
+                visit_lists(d.anodes, e, min(e + 32, e1), d.mptr, d.mlist, [&](i32 l) {
                     u32 h;
                     if (C.add(l, h)) {
                         const int f = atomicAdd(&sfill[w], 1);
@@ -540,7 +493,7 @@ __global__ void __launch_bounds__(BLK_WARPS * 32) pairs_block(const __grid_const
         const i64 e0 = d.aptr[k], e1 = d.aptr[k + 1], step = member_chunk(e1 - e0, BLK_WARPS);
         for (i64 e = e0 + w * step; e < e1; e += BLK_WARPS * step) {
             if (*(volatile int *)&over) break;
-            visit_partners(d, e, min(e + step, e1), [&](i32 l) {
+            visit_lists(d.anodes, e, min(e + step, e1), d.mptr, d.mlist, [&](i32 l) {
                 u32 h;
                 if (C.add(l, h)) {
                     const int f = atomicAdd(&fill, 1);
@@ -597,7 +550,7 @@ __global__ void __launch_bounds__(GLB_WARPS * 32) pairs_global(const __grid_cons
         unsigned int *fill = a.tfill + r;
         const i64 e0 = d.aptr[k], e1 = d.aptr[k + 1], step = member_chunk(e1 - e0, GLB_WARPS);
         for (i64 e = e0 + w * step; e < e1; e += GLB_WARPS * step)
-            visit_partners(d, e, min(e + step, e1), [&](i32 l) {
+            visit_lists(d.anodes, e, min(e + step, e1), d.mptr, d.mlist, [&](i32 l) {
                 u32 h;
                 if (C.add(l, h)) used[atomicAdd(fill, 1u)] = (i32)h;
             });
