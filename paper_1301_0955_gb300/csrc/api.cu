@@ -79,12 +79,6 @@ __global__ void sum_unit_stats(const i64 *ustat, const i32 *ulen, const i32 *ust
     }
 }
 
-// After a scale's dedup: unit j's list is its community's list.
-__global__ void point_units(const i32 *seed2comm, const i64 *comm_ptr, i64 N, i64 *uoff) {
-    for (i64 j = (i64)blockIdx.x * blockDim.x + threadIdx.x; j < N; j += (i64)gridDim.x * blockDim.x)
-        uoff[j] = comm_ptr[seed2comm[j]];
-}
-
 __global__ void gather_lists(const i64 *uoff, const i32 *ulen, const i64 *dst_ptr, const i32 *nodes, i64 N,
                              i32 *dst) {
     const int lane = threadIdx.x & 31;
@@ -636,15 +630,9 @@ int run_impl(mscd_ctx *c, int32_t graph_id, const double *alphas, int32_t n_scal
             dedup_ev.push_back({d0, d1});
             cudaEventRecord(d0, st);
             c->scales.resize(n_scales);
-            for (int32_t s = s0; s < s1 && rc == MSCD_OK; ++s) {
-                snprintf(stage, sizeof(stage), "dedup of scale %d", s);
-                rc = dedup_scale(c->uoff + s * N, c->ulen + s * N, c->uhash + s * N, c->uf + s * N,
-                                 c->pipe.out_nodes, N, &c->scales[s], st);
-                if (rc == MSCD_OK && N > 0) {
-                    point_units<<<152 * 4, 256, 0, st>>>(c->scales[s].seed2comm, c->scales[s].comm_ptr, N,
-                                                          c->uoff + s * N); note_launch();
-                }
-            }
+            snprintf(stage, sizeof(stage), "dedup of scales %d..%d", s0, s1 - 1);
+            rc = dedup_scales(c->uoff + s0 * N, c->ulen + s0 * N, c->uhash + s0 * N, c->uf + s0 * N,
+                              c->pipe.out_nodes, N, s1 - s0, c->scales.data() + s0, st);
             cudaEventRecord(d1, st);
         }
         s0 = s1;

@@ -10,13 +10,19 @@ struct ScaleResult {
     double *comm_f = nullptr;  // [n_comms]
     i32 *seed2comm = nullptr;  // [n_seeds]
     u64 *comm_hash = nullptr;  // [n_comms] hash of the member list
+    // scales deduplicated together keep their arrays in one block, which the
+    // first of them owns (the others are `shared`); else each array is its own
+    void *block = nullptr;
+    bool shared = false;
 };
 
 void scale_result_free(ScaleResult *r);
 
-// Units of one scale: uoff/ulen/uhash/uf indexed 0..N-1 (seed order), lists in nodes.
-int dedup_scale(const i64 *uoff, const i32 *ulen, const u64 *uhash, const double *uf, const i32 *nodes, i64 N,
-                ScaleResult *out, cudaStream_t st);
+// S scales of N units each, scale by scale (uoff, ulen, uhash and uf in seed
+// order), lists in nodes.  uoff then points into the results: unit j of scale s
+// has its list at out[s].comm_nodes + uoff[s * N + j].
+int dedup_scales(i64 *uoff, const i32 *ulen, const u64 *uhash, const double *uf, const i32 *nodes, i64 N, int32_t S,
+                 ScaleResult *out, cudaStream_t st);
 
 // Overlapping NMI between every two successive ones of S deduplicated
 // community sets over n nodes: nmi[s * P + p] between sets s and s + 1 for each

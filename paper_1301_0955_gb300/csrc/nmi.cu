@@ -38,12 +38,16 @@
 // integers), so the value does not depend on the order of the additions.
 //
 // The terms h(c/n) come from a table over c (binary64 logarithms cost some
-// 2,700 cycles each here, and a candidate needs six).  All the pairs of a run
-// are queued without waiting; only where a scale has more communities than a
-// CTA's table holds does the host look at the counters of a pair.
+// 2,700 cycles each here, and a candidate needs six).  A pair of scales is too
+// little work for the chip and a launch costs more than most pairs, so each
+// step is one launch over all the pairs of a run (as many as a bounded scratch
+// holds); only where a scale has more communities than a CTA's table holds
+// does the host look at the counters.
 // Stability of the 1-of-8 run of the 100,000-node graph (19 pairs): 55 ms with
-// a member at a time, logarithms per candidate and merges of sorted lists for
-// the disjoint pairs, now 9.5; of the 1,000-node graph (7 pairs) 3.7 and 1.0.
+// a member at a time, logarithms per candidate, merges of sorted lists for
+// the disjoint pairs and pair after pair, 9.5 pair after pair, now 3.0; of the
+// 1,000-node graph (7 pairs) 3.7, 1.0 and 0.26; of 20 scales of the
+// 10,000-node one 16.5, 4.2 and 0.48.
 //
 // A graph that is a disjoint union of parts (independent graphs batched as
 // one) gets one NMI per part: a community lies inside one part (growth never
@@ -111,9 +115,33 @@ __device__ __forceinline__ unsigned long long min_bits(double v) {
     return (unsigned long long)__double_as_longlong(v > 0.0 ? v : 0.0);
 }
 
-__global__ void count_memberships(const i32 *nodes, i64 m, i32 *cnt) {
-    for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (i64)gridDim.x * blockDim.x)
-        atomicAdd(&cnt[nodes[e]], 1);
+// Part of every community (that of its first member; a community never spans
+// parts), that part's node count and its place in the table of terms.
+struct CommParts {
+    i32 *cp;
+    i64 *cn;
+    i64 *ct;
+};
+
+// One scale's communities, and what its pairs with its neighbours share: the
+// communities' parts and the node -> communities lists.
+struct Scale {
+    const i64 *ptr;
+    const i32 *nodes;
+    const u64 *hash;
+    i64 C, m;
+    CommParts parts;
+    i32 *mcnt;    // [n] communities of a node
+    i32 *cursor;  // [n]
+    i64 *mptr;    // node u's are mlist[mptr[u]..mptr[u+1])
+    i32 *mlist;
+};
+
+// Kernels over scales: blockIdx.y is the scale.
+__global__ void count_memberships(const Scale *scales) {
+    const Scale &x = scales[blockIdx.y];
+    for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < x.m; e += (i64)gridDim.x * blockDim.x)
+        atomicAdd(&x.mcnt[x.nodes[e]], 1);
 }
 
 __global__ void widen_i32(const i32 *a, i64 n, i64 *b) {
@@ -121,115 +149,52 @@ __global__ void widen_i32(const i32 *a, i64 n, i64 *b) {
 }
 
 // Warp per community l: append l to the list of each member.
-__global__ void fill_memberships(const i64 *cptr, const i32 *nodes, i64 C, const i64 *mptr, i32 *cursor, i32 *mlist) {
+__global__ void fill_memberships(const Scale *scales) {
+    const Scale &x = scales[blockIdx.y];
     const int lane = threadIdx.x & 31;
     const i64 warps = (i64)gridDim.x * (blockDim.x >> 5);
-    for (i64 l = (i64)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); l < C; l += warps)
-        for (i64 e = cptr[l] + lane; e < cptr[l + 1]; e += 32) {
-            const i32 u = nodes[e];
-            mlist[mptr[u] + atomicAdd(&cursor[u], 1)] = (i32)l;
+    for (i64 l = (i64)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); l < x.C; l += warps)
+        for (i64 e = x.ptr[l] + lane; e < x.ptr[l + 1]; e += 32) {
+            const i32 u = x.nodes[e];
+            x.mlist[x.mptr[u] + atomicAdd(&x.cursor[u], 1)] = (i32)l;
         }
 }
 
-// Hash table of community list hashes (0 = empty bucket; list hashes are never 0).
-__global__ void hash_insert(const u64 *chash, i64 C, u64 *tkey, i32 *tval, i64 tmask) {
-    for (i64 l = (i64)blockIdx.x * blockDim.x + threadIdx.x; l < C; l += (i64)gridDim.x * blockDim.x) {
-        i64 h = (i64)(chash[l] & (u64)tmask);
-        for (i64 p = 0; p <= tmask; ++p) {
-            if (atomicCAS((unsigned long long *)&tkey[h], 0ull, (unsigned long long)chash[l]) == 0ull) {
-                tval[h] = (i32)l;
-                break;
-            }
-            h = (h + 1) & tmask;
-        }
-    }
-}
-
-// Warp per X_k: an identical Y_l (same hash, same list) zeroes both.
-__global__ void match_identical(const i64 *xptr, const i32 *xnodes, const u64 *xhash, i64 CX, const i64 *yptr,
-                                const i32 *ynodes, const u64 *tkey, const i32 *tval, i64 tmask,
-                                unsigned char *zeroX, unsigned char *zeroY) {
-    const int lane = threadIdx.x & 31;
-    const i64 warps = (i64)gridDim.x * (blockDim.x >> 5);
-    for (i64 k = (i64)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); k < CX; k += warps) {
-        const u64 key = xhash[k];
-        const i64 sx = xptr[k + 1] - xptr[k];
-        i64 h = (i64)(key & (u64)tmask);
-        for (i64 p = 0; p <= tmask; ++p) {
-            const u64 tk = tkey[h];
-            if (tk == 0ull) break;
-            if (tk == key) {
-                const i32 l = tval[h];
-                bool eq = yptr[l + 1] - yptr[l] == sx;
-                if (eq) {
-                    const i32 *a = xnodes + xptr[k], *b = ynodes + yptr[l];
-                    bool diff = false;
-                    for (i64 i = lane; i < sx; i += 32) diff |= a[i] != b[i];
-                    eq = !__any_sync(FULL_MASK, diff);
-                }
-                if (eq) {
-                    if (lane == 0) {
-                        zeroX[k] = 1;
-                        zeroY[l] = 1;
-                    }
-                    break;
-                }
-            }
-            h = (h + 1) & tmask;
-        }
-    }
-}
-
-// Part of every community (that of its first member; a community never spans
-// parts), that part's node count and its place in the table of terms.  No
-// offsets: one part of n nodes.
-struct CommParts {
-    i32 *cp = nullptr;
-    i64 *cn = nullptr;
-    i64 *ct = nullptr;
-};
-
-__global__ void comm_parts(const i64 *ptr, const i32 *nodes, i64 C, const i64 *off, i32 n_parts, i64 n, CommParts out) {
-    for (i64 l = (i64)blockIdx.x * blockDim.x + threadIdx.x; l < C; l += (i64)gridDim.x * blockDim.x) {
+// No offsets: one part of n nodes.
+__global__ void comm_parts(const Scale *scales, const i64 *off, i32 n_parts, i64 n) {
+    const Scale &x = scales[blockIdx.y];
+    for (i64 l = (i64)blockIdx.x * blockDim.x + threadIdx.x; l < x.C; l += (i64)gridDim.x * blockDim.x) {
         if (!off) {
-            out.cp[l] = 0;
-            out.cn[l] = n;
-            out.ct[l] = 0;
+            x.parts.cp[l] = 0;
+            x.parts.cn[l] = n;
+            x.parts.ct[l] = 0;
             continue;
         }
-        const i64 u = nodes[ptr[l]];
+        const i64 u = x.nodes[x.ptr[l]];
         i32 lo = 0, hi = n_parts - 1;  // last part with off[p] <= u
         while (lo < hi) {
             const i32 mid = (lo + hi + 1) >> 1;
             if (off[mid] <= u) lo = mid;
             else hi = mid - 1;
         }
-        out.cp[l] = lo;
-        out.cn[l] = off[lo + 1] - off[lo];
-        out.ct[l] = off[lo] + lo;
+        x.parts.cp[l] = lo;
+        x.parts.cn[l] = off[lo + 1] - off[lo];
+        x.parts.ct[l] = off[lo] + lo;
     }
 }
 
 __device__ __forceinline__ u32 hash_comm(i32 l) { return (u32)l * 0x9E3779B1u; }
 
 // One direction of a pair of scales: H(A_k|B) for the communities of A
-// without an identical partner (the active ones).
+// without an identical partner (the active ones).  Directions 2p and 2p + 1
+// are those of pair p.
 struct Direction {
-    const i64 *aptr;
-    const i32 *anodes;
-    i64 CA;
-    CommParts ap;
-    const unsigned char *zero;  // has an identical partner
+    Scale A, B;
+    unsigned char *zero;        // per A community: has an identical partner
     i32 *active;
     unsigned long long *n_active;
     unsigned long long *best;   // per A community (bits of doubles)
     unsigned long long *amax;   // per part: the largest active A community
-    const i64 *bptr;
-    i64 CB;
-    CommParts bp;
-    const i32 *mcnt;            // node -> number of communities of B,
-    const i64 *mptr;            // node -> communities of B
-    const i32 *mlist;
     // B communities that can meet an active A community of their part in an
     // admitted disjoint pair, by part (boff), and the largest of each part
     i32 *big;
@@ -237,16 +202,20 @@ struct Direction {
     unsigned long long *bmax, *bcount, *bfill;
     i64 *spill, *spill2;        // positions in `active` left to the next tier
     unsigned long long *n_spill, *n_spill2;
+    // work counters of the tiers: communities are taken one at a time as warps
+    // or CTAs free up, since their costs differ by orders of magnitude
+    unsigned long long *next_warp, *next_block;
+    unsigned long long *sum, *count;  // per part: 128-bit sum, number of communities
+    u64 *tkey;                  // direction 2p: hash table of B's list hashes
+    i32 *tval;
+    i64 tmask;
 };
 
 struct PairArgs {
-    Direction d[2];
+    const Direction *d;  // on the device
+    int n;               // directions
     i32 P;
     const double *tab;
-    // work counters of the launches (zeroed before): communities are taken one
-    // at a time as warps or CTAs free up, since their costs differ by orders of
-    // magnitude; both directions share a launch
-    unsigned long long *next_warp, *next_block;
     // global tables of the last tier
     const i64 *toff;
     i32 *tkey, *tcnt;
@@ -255,9 +224,62 @@ struct PairArgs {
     unsigned long long *next_global;
 };
 
+// Hash table of B's community list hashes (0 = empty bucket; list hashes are
+// never 0).  blockIdx.y: the pair.
+__global__ void hash_insert(PairArgs a) {
+    const Direction &d = a.d[2 * blockIdx.y];
+    for (i64 l = (i64)blockIdx.x * blockDim.x + threadIdx.x; l < d.B.C; l += (i64)gridDim.x * blockDim.x) {
+        const u64 key = d.B.hash[l];
+        i64 h = (i64)(key & (u64)d.tmask);
+        for (i64 p = 0; p <= d.tmask; ++p) {
+            if (atomicCAS((unsigned long long *)&d.tkey[h], 0ull, (unsigned long long)key) == 0ull) {
+                d.tval[h] = (i32)l;
+                break;
+            }
+            h = (h + 1) & d.tmask;
+        }
+    }
+}
+
+// Warp per A_k: an identical B_l (same hash, same list) zeroes both.
+// blockIdx.y: the pair.
+__global__ void match_identical(PairArgs a) {
+    const Direction &d = a.d[2 * blockIdx.y];
+    unsigned char *zeroB = a.d[2 * blockIdx.y + 1].zero;
+    const int lane = threadIdx.x & 31;
+    const i64 warps = (i64)gridDim.x * (blockDim.x >> 5);
+    for (i64 k = (i64)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); k < d.A.C; k += warps) {
+        const u64 key = d.A.hash[k];
+        const i64 sx = d.A.ptr[k + 1] - d.A.ptr[k];
+        i64 h = (i64)(key & (u64)d.tmask);
+        for (i64 p = 0; p <= d.tmask; ++p) {
+            const u64 tk = d.tkey[h];
+            if (tk == 0ull) break;
+            if (tk == key) {
+                const i32 l = d.tval[h];
+                bool eq = d.B.ptr[l + 1] - d.B.ptr[l] == sx;
+                if (eq) {
+                    const i32 *x = d.A.nodes + d.A.ptr[k], *y = d.B.nodes + d.B.ptr[l];
+                    bool diff = false;
+                    for (i64 i = lane; i < sx; i += 32) diff |= x[i] != y[i];
+                    eq = !__any_sync(FULL_MASK, diff);
+                }
+                if (eq) {
+                    if (lane == 0) {
+                        d.zero[k] = 1;
+                        zeroB[l] = 1;
+                    }
+                    break;
+                }
+            }
+            h = (h + 1) & d.tmask;
+        }
+    }
+}
+
 // h(c/n) for the part of A's community k.
 __device__ __forceinline__ Terms terms_of(const PairArgs &a, const Direction &d, i32 k) {
-    return {a.tab ? a.tab + d.ap.ct[k] : nullptr, 1.0 / (double)d.ap.cn[k]};
+    return {a.tab ? a.tab + d.A.parts.ct[k] : nullptr, 1.0 / (double)d.A.parts.cn[k]};
 }
 
 // Initial minima: 0 for communities with an identical partner, else H(C)
@@ -265,14 +287,14 @@ __device__ __forceinline__ Terms terms_of(const PairArgs &a, const Direction &d,
 // of them per part.  blockIdx.y: the direction (also below).
 __global__ void init_best(PairArgs a) {
     const Direction &d = a.d[blockIdx.y];
-    for (i64 l = (i64)blockIdx.x * blockDim.x + threadIdx.x; l < d.CA; l += (i64)gridDim.x * blockDim.x) {
+    for (i64 l = (i64)blockIdx.x * blockDim.x + threadIdx.x; l < d.A.C; l += (i64)gridDim.x * blockDim.x) {
         if (d.zero[l]) {
             d.best[l] = 0ull;
         } else {
-            const i64 s = d.aptr[l + 1] - d.aptr[l];
-            d.best[l] = min_bits(entropy(s, d.ap.cn[l], terms_of(a, d, (i32)l)));
+            const i64 s = d.A.ptr[l + 1] - d.A.ptr[l];
+            d.best[l] = min_bits(entropy(s, d.A.parts.cn[l], terms_of(a, d, (i32)l)));
             d.active[atomicAdd(d.n_active, 1ull)] = (i32)l;
-            atomicMax(&d.amax[d.ap.cp[l]], (unsigned long long)s);
+            atomicMax(&d.amax[d.A.parts.cp[l]], (unsigned long long)s);
         }
     }
 }
@@ -281,10 +303,10 @@ __global__ void init_best(PairArgs a) {
 // community of that part).  fill = 0 counts them per part, fill = 1 lists them.
 __global__ void list_big(PairArgs a, int fill) {
     const Direction &d = a.d[blockIdx.y];
-    for (i64 l = (i64)blockIdx.x * blockDim.x + threadIdx.x; l < d.CB; l += (i64)gridDim.x * blockDim.x) {
-        const i32 p = d.bp.cp[l];
-        const i64 amax = (i64)d.amax[p], s = d.bptr[l + 1] - d.bptr[l];
-        if (amax == 0 || 2 * (s + amax) <= d.bp.cn[l]) continue;
+    for (i64 l = (i64)blockIdx.x * blockDim.x + threadIdx.x; l < d.B.C; l += (i64)gridDim.x * blockDim.x) {
+        const i32 p = d.B.parts.cp[l];
+        const i64 amax = (i64)d.amax[p], s = d.B.ptr[l + 1] - d.B.ptr[l];
+        if (amax == 0 || 2 * (s + amax) <= d.B.parts.cn[l]) continue;
         if (fill) {
             d.big[d.boff[p] + (i64)atomicAdd(&d.bfill[p], 1ull)] = (i32)l;
         } else {
@@ -356,19 +378,19 @@ struct Counts {
 template <class B>
 __device__ __forceinline__ double least_candidate(const PairArgs &a, const Direction &d, i32 k, const Counts &C, int nf,
                                                   B bucket, int rank, int size) {
-    const i64 sa = d.aptr[k + 1] - d.aptr[k], n = d.ap.cn[k];
+    const i64 sa = d.A.ptr[k + 1] - d.A.ptr[k], n = d.A.parts.cn[k];
     const Terms H = terms_of(a, d, k);
     double bx = __builtin_huge_val();
     for (int t = rank; t < nf; t += size) {
         const u32 h = bucket(t);
         const i32 l = C.keys[h];
-        bx = min(bx, cond_candidate(C.cnts[h], sa, d.bptr[l + 1] - d.bptr[l], n, H));
+        bx = min(bx, cond_candidate(C.cnts[h], sa, d.B.ptr[l + 1] - d.B.ptr[l], n, H));
     }
-    const i32 p = d.ap.cp[k];
+    const i32 p = d.A.parts.cp[k];
     if (2 * (sa + (i64)d.bmax[p]) > n)
         for (i64 j = d.boff[p] + rank; j < d.boff[p + 1]; j += size) {
             const i32 l = d.big[j];
-            const i64 sb = d.bptr[l + 1] - d.bptr[l];
+            const i64 sb = d.B.ptr[l + 1] - d.B.ptr[l];
             if (2 * (sa + sb) > n && !C.has(l)) bx = min(bx, cond_candidate(0, sa, sb, n, H));
         }
     return bx;
@@ -396,26 +418,30 @@ __global__ void __launch_bounds__(NMI_WARPS * 32) pairs_warp(const __grid_consta
         C.cnts[t] = 0;
     }
     __syncwarp();
-    const i64 n0 = (i64)*a.d[0].n_active, n1 = (i64)*a.d[1].n_active;
-    for (;;) {
+    // the directions in turn, each warp from another one on
+    int dir = (int)((blockIdx.x * NMI_WARPS + w) % a.n), left = a.n;
+    while (left > 0) {
+        const Direction &d = a.d[dir];
         unsigned long long qq = 0;
-        if (lane == 0) qq = atomicAdd(a.next_warp, 1ull);
-        i64 q = (i64)__shfl_sync(FULL_MASK, qq, 0);
-        if (q >= n0 + n1) break;
-        const Direction &d = a.d[q >= n0 ? 1 : 0];
-        if (q >= n0) q -= n0;
+        if (lane == 0) qq = atomicAdd(d.next_warp, 1ull);
+        const i64 q = (i64)__shfl_sync(FULL_MASK, qq, 0);
+        if (q >= (i64)*d.n_active) {
+            if (++dir == a.n) dir = 0;
+            --left;
+            continue;
+        }
         const i32 k = d.active[q];
-        const i64 e0 = d.aptr[k], e1 = d.aptr[k + 1];
+        const i64 e0 = d.A.ptr[k], e1 = d.A.ptr[k + 1];
         i64 entries = 0;
 #pragma unroll 4
-        for (i64 e = e0 + lane; e < e1; e += 32) entries += d.mcnt[d.anodes[e]];
+        for (i64 e = e0 + lane; e < e1; e += 32) entries += d.B.mcnt[d.A.nodes[e]];
         for (int o = 16; o; o >>= 1) entries += __shfl_xor_sync(FULL_MASK, entries, o);
         bool over = entries > WARP_ENTRIES;
         if (!over) {
             if (lane == 0) sfill[w] = 0;
             __syncwarp();
             for (i64 e = e0; e < e1 && !over; e += 32) {
-                visit_lists(d.anodes, e, min(e + 32, e1), d.mptr, d.mlist, [&](i32 l) {
+                visit_lists(d.A.nodes, e, min(e + 32, e1), d.B.mptr, d.B.mlist, [&](i32 l) {
                     u32 h;
                     if (C.add(l, h)) {
                         const int f = atomicAdd(&sfill[w], 1);
@@ -470,30 +496,40 @@ __global__ void __launch_bounds__(BLK_WARPS * 32) pairs_block(const __grid_const
     __shared__ double wmin[BLK_WARPS];
     __shared__ i64 rnext;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const i64 n0 = (i64)*a.d[0].n_spill, n1 = (i64)*a.d[1].n_spill;
-    if (n0 + n1 == 0) return;
-    for (int t = threadIdx.x; t < BLK_TABLE; t += BLK_WARPS * 32) {
-        C.keys[t] = -1;
-        C.cnts[t] = 0;
-    }
-    for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            rnext = (i64)atomicAdd(a.next_block, 1ull);
-            fill = 0;
-            over = 0;
+    bool clear = false;  // the table has been cleared
+    int dir = (int)(blockIdx.x % a.n), left = a.n;
+    while (left > 0) {
+        const Direction &d = a.d[dir];
+        const i64 ns = (i64)*d.n_spill;
+        if (ns > 0) {
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                rnext = (i64)atomicAdd(d.next_block, 1ull);
+                fill = 0;
+                over = 0;
+            }
+            __syncthreads();
         }
-        __syncthreads();
-        i64 r = rnext;
-        if (r >= n0 + n1) break;
-        const Direction &d = a.d[r >= n0 ? 1 : 0];
-        if (r >= n0) r -= n0;
+        const i64 r = ns > 0 ? rnext : 0;
+        if (r >= ns) {
+            if (++dir == a.n) dir = 0;
+            --left;
+            continue;
+        }
+        if (!clear) {
+            for (int t = threadIdx.x; t < BLK_TABLE; t += BLK_WARPS * 32) {
+                C.keys[t] = -1;
+                C.cnts[t] = 0;
+            }
+            clear = true;
+            __syncthreads();
+        }
         const i64 q = d.spill[r];
         const i32 k = d.active[q];
-        const i64 e0 = d.aptr[k], e1 = d.aptr[k + 1], step = member_chunk(e1 - e0, BLK_WARPS);
+        const i64 e0 = d.A.ptr[k], e1 = d.A.ptr[k + 1], step = member_chunk(e1 - e0, BLK_WARPS);
         for (i64 e = e0 + w * step; e < e1; e += BLK_WARPS * step) {
             if (*(volatile int *)&over) break;
-            visit_lists(d.anodes, e, min(e + step, e1), d.mptr, d.mlist, [&](i32 l) {
+            visit_lists(d.A.nodes, e, min(e + step, e1), d.B.mptr, d.B.mlist, [&](i32 l) {
                 u32 h;
                 if (C.add(l, h)) {
                     const int f = atomicAdd(&fill, 1);
@@ -548,9 +584,9 @@ __global__ void __launch_bounds__(GLB_WARPS * 32) pairs_global(const __grid_cons
         const Counts C = {a.tkey + a.toff[r], a.tcnt + a.toff[r], (u32)(a.toff[r + 1] - a.toff[r] - 1)};
         i32 *used = a.tused + a.toff[r];
         unsigned int *fill = a.tfill + r;
-        const i64 e0 = d.aptr[k], e1 = d.aptr[k + 1], step = member_chunk(e1 - e0, GLB_WARPS);
+        const i64 e0 = d.A.ptr[k], e1 = d.A.ptr[k + 1], step = member_chunk(e1 - e0, GLB_WARPS);
         for (i64 e = e0 + w * step; e < e1; e += GLB_WARPS * step)
-            visit_lists(d.anodes, e, min(e + step, e1), d.mptr, d.mlist, [&](i32 l) {
+            visit_lists(d.A.nodes, e, min(e + step, e1), d.B.mptr, d.B.mlist, [&](i32 l) {
                 u32 h;
                 if (C.add(l, h)) used[atomicAdd(fill, 1u)] = (i32)h;
             });
@@ -576,15 +612,16 @@ __global__ void __launch_bounds__(GLB_WARPS * 32) pairs_global(const __grid_cons
 
 // Table size of each community of the last tier: 2 * min(incidences, |B|)
 // rounded up to a power of two.
-__global__ void spill_sizes(const i64 *list, i64 nk, Direction d, i64 *tsz) {
+__global__ void spill_sizes(const i64 *list, i64 nk, const Direction *dp, i64 *tsz) {
+    const Direction &d = *dp;
     const int lane = threadIdx.x & 31;
     const i64 warps = (i64)gridDim.x * (blockDim.x >> 5);
     for (i64 r = (i64)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < nk; r += warps) {
         const i32 k = d.active[list[r]];
         i64 s = 0;
-        for (i64 e = d.aptr[k] + lane; e < d.aptr[k + 1]; e += 32) s += d.mcnt[d.anodes[e]];
+        for (i64 e = d.A.ptr[k] + lane; e < d.A.ptr[k + 1]; e += 32) s += d.B.mcnt[d.A.nodes[e]];
         for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(FULL_MASK, s, o);
-        s = min(s, d.CB);
+        s = min(s, d.B.C);
         i64 t = 2;
         while (t < 2 * s) t <<= 1;
         if (lane == 0) tsz[r] = t;
@@ -593,18 +630,17 @@ __global__ void spill_sizes(const i64 *list, i64 nk, Direction d, i64 *tsz) {
 
 // Normalised term H(A_k|B) / H(A_k) in [0, 1] (the minimum never exceeds its
 // initial value H(A_k), computed the same way), added to its part's total as
-// an integer multiple of 2^-62 in 128 bits.  acc: per part, the two
-// directions' sums (low word, carries), then their counts.  One part: the
+// an integer multiple of 2^-62 in 128 bits (low word, carries).  One part: the
 // warps' sums are added first (every community on one address otherwise).
-__global__ void normalise_sum(PairArgs a, unsigned long long *acc) {
+__global__ void normalise_sum(PairArgs a) {
     const Direction &d = a.d[blockIdx.y];
-    unsigned long long *sum = acc + (size_t)blockIdx.y * 2 * a.P, *count = acc + (size_t)(4 + blockIdx.y) * a.P;
+    unsigned long long *sum = d.sum, *count = d.count;
     const i64 stride = (i64)gridDim.x * blockDim.x;
-    for (i64 k0 = (i64)blockIdx.x * blockDim.x; k0 < d.CA; k0 += stride) {
+    for (i64 k0 = (i64)blockIdx.x * blockDim.x; k0 < d.A.C; k0 += stride) {
         const i64 k = k0 + threadIdx.x;
         unsigned long long q = 0;
-        if (k < d.CA) {
-            const double H = entropy(d.aptr[k + 1] - d.aptr[k], d.ap.cn[k], terms_of(a, d, (i32)k));
+        if (k < d.A.C) {
+            const double H = entropy(d.A.ptr[k + 1] - d.A.ptr[k], d.A.parts.cn[k], terms_of(a, d, (i32)k));
             const double t = H > 0.0 ? __longlong_as_double((long long)d.best[k]) / H : 0.0;
             q = (unsigned long long)__double2ll_rn(fmin(fmax(t, 0.0), 1.0) * 0x1p62);
         }
@@ -615,15 +651,15 @@ __global__ void normalise_sum(PairArgs a, unsigned long long *acc) {
                 lo += l2;
                 hi += h2 + (lo < l2 ? 1ull : 0ull);
             }
-            const int live = __popc(__ballot_sync(FULL_MASK, k < d.CA));
+            const int live = __popc(__ballot_sync(FULL_MASK, k < d.A.C));
             if ((threadIdx.x & 31) == 0 && live) {
                 const unsigned long long old = atomicAdd(&sum[0], lo);
                 hi += old + lo < old ? 1ull : 0ull;
                 if (hi) atomicAdd(&sum[1], hi);
                 atomicAdd(&count[0], (unsigned long long)live);
             }
-        } else if (k < d.CA) {
-            const i32 p = d.ap.cp[k];
+        } else if (k < d.A.C) {
+            const i32 p = d.A.parts.cp[k];
             const unsigned long long old = atomicAdd(&sum[2 * p], q);
             if (old + q < old) atomicAdd(&sum[2 * p + 1], 1ull);
             atomicAdd(&count[p], 1ull);
@@ -638,68 +674,16 @@ int dev_alloc(T **p, i64 count, cudaStream_t st) {
 
 const unsigned GB = 152 * 16;
 constexpr i64 TERMS_MAX = (i64)1 << 26;  // nodes up to which the terms are tabled (8 bytes each)
+constexpr size_t CHUNK_SCRATCH = (size_t)1 << 30;  // scratch of the scales handled together, at most (or two scales)
+constexpr int CHUNK_SCALES = 16384;  // two directions a pair on a grid's y axis
 
 // CTAs of 256 threads for m threads of work.
 unsigned grid_of(i64 m) { return (unsigned)std::max<i64>(1, std::min<i64>((m + 255) / 256, GB)); }
 
-// node -> communities map of B.
-struct Memberships {
-    i32 *cnt = nullptr, *list = nullptr;
-    i64 *ptr = nullptr;
-};
-
-int build_memberships(const ScaleResult &B, i64 n, Memberships *M, cudaStream_t st) {
-    i32 *cursor = nullptr;
-    i64 *tmp = nullptr;
-    int rc = MSCD_OK;
-    do {
-        if ((rc = dev_alloc(&M->cnt, 2 * n, st))) break;
-        cursor = M->cnt + n;
-        if ((rc = dev_alloc(&M->ptr, n + 1, st))) break;
-        if ((rc = dev_alloc(&M->list, B.n_nodes, st))) break;
-        if ((rc = dev_alloc(&tmp, n + 1, st))) break;
-        if ((rc = cuda_status(cudaMemsetAsync(M->cnt, 0, 2 * n * sizeof(i32), st)))) break;
-        count_memberships<<<grid_of(B.n_nodes), 256, 0, st>>>(B.comm_nodes, B.n_nodes, M->cnt); note_launch();
-        widen_i32<<<grid_of(n), 256, 0, st>>>(M->cnt, n, tmp); note_launch();
-        if ((rc = scan_exclusive_i64(tmp, M->ptr, n, M->ptr + n, st))) break;
-        fill_memberships<<<grid_of(32 * B.n_comms), 256, 0, st>>>(B.comm_ptr, B.comm_nodes, B.n_comms, M->ptr, cursor,
-                                                                  M->list); note_launch();
-    } while (0);
-    cudaFreeAsync(tmp, st);
-    return rc;
-}
-
-// What the pairs of a scale with its neighbours share.
-struct ScaleData {
-    CommParts parts;
-    Memberships members;
-};
-
-void free_scale(ScaleData *s, cudaStream_t st) {
-    cudaFreeAsync(s->parts.cp, st);
-    cudaFreeAsync(s->parts.cn, st);
-    cudaFreeAsync(s->parts.ct, st);
-    cudaFreeAsync(s->members.cnt, st);
-    cudaFreeAsync(s->members.ptr, st);
-    cudaFreeAsync(s->members.list, st);
-    *s = ScaleData{};
-}
-
-int build_scale(const ScaleResult &R, i64 n, const i64 *part_off, int32_t P, ScaleData *s, cudaStream_t st) {
-    int rc = dev_alloc(&s->parts.cp, R.n_comms, st);
-    if (!rc) rc = dev_alloc(&s->parts.cn, R.n_comms, st);
-    if (!rc) rc = dev_alloc(&s->parts.ct, R.n_comms, st);
-    if (rc) return rc;
-    comm_parts<<<grid_of(R.n_comms), 256, 0, st>>>(R.comm_ptr, R.comm_nodes, R.n_comms, part_off, P, n, s->parts);
-    note_launch();
-    return build_memberships(R, n, &s->members, st);
-}
-
 // The last tier of one direction: a global table per community, 2
 // min(incidences, |B|) entries; communities go in chunks whose tables fit a
 // bounded scratch (a single table is at most 2^(1+ceil log2 |B|) entries).
-int global_tier(PairArgs a, int dir, i64 nk, cudaStream_t st) {
-    const Direction &d = a.d[dir];
+int global_tier(PairArgs a, int dir, const Direction &d, i64 nk, cudaStream_t st) {
     i64 *tsz = nullptr, *toff = nullptr;
     i32 *tables = nullptr;
     unsigned int *tfill = nullptr;
@@ -707,7 +691,7 @@ int global_tier(PairArgs a, int dir, i64 nk, cudaStream_t st) {
     do {
         if ((rc = dev_alloc(&tsz, nk + 1, st))) break;
         if ((rc = dev_alloc(&toff, nk + 1, st))) break;
-        spill_sizes<<<GB, 256, 0, st>>>(d.spill2, nk, d, tsz); note_launch();
+        spill_sizes<<<GB, 256, 0, st>>>(d.spill2, nk, a.d + dir, tsz); note_launch();
         std::vector<i64> hs(nk);
         if ((rc = cuda_status(cudaMemcpyAsync(hs.data(), tsz, nk * sizeof(i64), cudaMemcpyDeviceToHost, st)))) break;
         if ((rc = cuda_status(cudaStreamSynchronize(st)))) break;
@@ -758,107 +742,164 @@ int global_tier(PairArgs a, int dir, i64 nk, cudaStream_t st) {
     return rc;
 }
 
-// One pair of scales into acc (6 P words, zero).  Waits for the stream only
-// where a community may meet more partners than a CTA's table holds.
-int pair_terms(const ScaleResult &X, const ScaleResult &Y, const ScaleData &DX, const ScaleData &DY, int32_t P,
-               const double *tab, unsigned long long *acc, cudaStream_t st) {
-    const i64 C[2] = {X.n_comms, Y.n_comms};
-    i64 T = 2;
-    while (T < 2 * C[1]) T <<= 1;
-    // one allocation: what starts as zero first
-    enum { N_ACTIVE = 0, N_SPILL = 2, N_SPILL2 = 4, NEXT_WARP = 6, NEXT_BLOCK, NEXT_GLOBAL, COUNTERS };
+// Sub-allocations of one block of device memory.
+struct Rooms {
     size_t at = 0;
-    auto room = [&](size_t bytes) {
+    size_t take(size_t bytes) {
         const size_t o = at;
         at += (bytes + 15) & ~(size_t)15;
         return o;
-    };
-    const size_t o_cnt = room(COUNTERS * 8), o_part = room(8 * (size_t)P * 8), o_tkey = room((size_t)T * 8);
-    const size_t o_zero[2] = {room((size_t)C[0]), room((size_t)C[1])};
-    const size_t zeroed = at;
-    const size_t o_tval = room((size_t)T * 4), o_boff = room(2 * ((size_t)P + 1) * 8);
-    size_t o_best[2], o_act[2], o_big[2], o_sp[2], o_sp2[2];
-    for (int i = 0; i < 2; ++i) {
-        o_best[i] = room((size_t)C[i] * 8);
-        o_act[i] = room((size_t)C[i] * 4);
-        o_big[i] = room((size_t)C[1 - i] * 4);
-        o_sp[i] = room((size_t)C[i] * 8);
-        o_sp2[i] = room((size_t)C[i] * 8);
+    }
+};
+
+// The pairs of the successive scales sc[0..ns) (each with communities) into
+// acc (6 P words per pair, zero): every step is one launch over all of them.
+// Waits for the stream only where a community may meet more partners than a
+// CTA's table holds.
+int chunk_terms(const ScaleResult *sc, int ns, i64 n, const i64 *part_off, int32_t P, const double *tab,
+                unsigned long long *acc, cudaStream_t st) {
+    const int np = ns - 1, nd = 2 * np;
+    i64 most = 0, most_m = 0;
+    for (int s = 0; s < ns; ++s) {
+        most = std::max(most, sc[s].n_comms);
+        most_m = std::max(most_m, sc[s].n_nodes);
+    }
+    // one block: what starts as zero first
+    Rooms R;
+    enum { N_ACTIVE, N_SPILL, N_SPILL2, NEXT_WARP, NEXT_BLOCK, COUNTERS };
+    const size_t o_cnt = R.take((size_t)(nd * COUNTERS + 1) * 8);  // counter c of direction i at c * nd + i
+    const size_t o_part = R.take((size_t)nd * 4 * P * 8);
+    const size_t o_mcnt = R.take((size_t)ns * n * 4), o_cursor = R.take((size_t)ns * n * 4);
+    std::vector<size_t> o_tkey(np), o_zero(nd);
+    std::vector<i64> T(np, 2);
+    for (int p = 0; p < np; ++p) {
+        while (T[p] < 2 * sc[p + 1].n_comms) T[p] <<= 1;
+        o_tkey[p] = R.take((size_t)T[p] * 8);
+        o_zero[2 * p] = R.take((size_t)sc[p].n_comms);
+        o_zero[2 * p + 1] = R.take((size_t)sc[p + 1].n_comms);
+    }
+    const size_t zeroed = R.at;
+    const size_t o_scales = R.take(ns * sizeof(Scale)), o_dirs = R.take(nd * sizeof(Direction));
+    const size_t o_boff = R.take((size_t)nd * (P + 1) * 8);
+    const size_t o_wide = R.take((size_t)ns * n * 8), o_mptr = R.take(((size_t)ns * n + 1) * 8);
+    i64 entries = 0;
+    for (int s = 0; s < ns; ++s) entries += sc[s].n_nodes;
+    const size_t o_mlist = R.take((size_t)entries * 4);
+    std::vector<Scale> scales(ns);
+    std::vector<Direction> dirs(nd);
+    std::vector<size_t> o_s(3 * ns), o_d(6 * nd);
+    for (int s = 0; s < ns; ++s) {
+        const size_t C = (size_t)sc[s].n_comms;
+        o_s[3 * s] = R.take(C * 4);
+        o_s[3 * s + 1] = R.take(C * 8);
+        o_s[3 * s + 2] = R.take(C * 8);
+    }
+    for (int i = 0; i < nd; ++i) {
+        const size_t CA = (size_t)sc[i / 2 + (i & 1)].n_comms, CB = (size_t)sc[i / 2 + 1 - (i & 1)].n_comms;
+        o_d[6 * i] = R.take(CA * 8);
+        o_d[6 * i + 1] = R.take(CA * 4);
+        o_d[6 * i + 2] = R.take(CB * 4);
+        o_d[6 * i + 3] = R.take(CA * 8);
+        o_d[6 * i + 4] = R.take(CA * 8);
+        o_d[6 * i + 5] = i & 1 ? 0 : R.take((size_t)T[i / 2] * 4);
     }
     unsigned char *mem = nullptr;
-    int rc = dev_alloc(&mem, (i64)at, st);
+    int rc = dev_alloc(&mem, (i64)R.at, st);
     if (rc) return rc;
     unsigned long long *cnt = (unsigned long long *)(mem + o_cnt), *part = (unsigned long long *)(mem + o_part);
-    PairArgs a{};
-    a.P = P;
-    a.tab = tab;
-    a.next_warp = cnt + NEXT_WARP;
-    a.next_block = cnt + NEXT_BLOCK;
-    a.next_global = cnt + NEXT_GLOBAL;
-    for (int i = 0; i < 2; ++i) {
-        const ScaleResult &A = i ? Y : X, &B = i ? X : Y;
-        const ScaleData &DA = i ? DY : DX, &DB = i ? DX : DY;
-        Direction &d = a.d[i];
-        d.aptr = A.comm_ptr;
-        d.anodes = A.comm_nodes;
-        d.CA = A.n_comms;
-        d.ap = DA.parts;
+    for (int s = 0; s < ns; ++s) {
+        Scale &x = scales[s];
+        x.ptr = sc[s].comm_ptr;
+        x.nodes = sc[s].comm_nodes;
+        x.hash = sc[s].comm_hash;
+        x.C = sc[s].n_comms;
+        x.m = sc[s].n_nodes;
+        x.parts = {(i32 *)(mem + o_s[3 * s]), (i64 *)(mem + o_s[3 * s + 1]), (i64 *)(mem + o_s[3 * s + 2])};
+        x.mcnt = (i32 *)(mem + o_mcnt) + (size_t)s * n;
+        x.cursor = (i32 *)(mem + o_cursor) + (size_t)s * n;
+        x.mptr = (i64 *)(mem + o_mptr) + (size_t)s * n;  // one scan over all scales: mptr[n] is the next one's first
+        x.mlist = (i32 *)(mem + o_mlist);
+    }
+    for (int i = 0; i < nd; ++i) {
+        Direction &d = dirs[i];
+        const int p = i / 2;
+        d.A = scales[p + (i & 1)];
+        d.B = scales[p + 1 - (i & 1)];
         d.zero = mem + o_zero[i];
-        d.active = (i32 *)(mem + o_act[i]);
-        d.n_active = cnt + N_ACTIVE + i;
-        d.best = (unsigned long long *)(mem + o_best[i]);
+        unsigned long long **counters[] = {&d.n_active, &d.n_spill, &d.n_spill2, &d.next_warp, &d.next_block};
+        for (int c = 0; c < COUNTERS; ++c) *counters[c] = cnt + c * nd + i;
         d.amax = part + (size_t)(4 * i) * P;
         d.bmax = part + (size_t)(4 * i + 1) * P;
         d.bcount = part + (size_t)(4 * i + 2) * P;
         d.bfill = part + (size_t)(4 * i + 3) * P;
-        d.bptr = B.comm_ptr;
-        d.CB = B.n_comms;
-        d.bp = DB.parts;
-        d.mcnt = DB.members.cnt;
-        d.mptr = DB.members.ptr;
-        d.mlist = DB.members.list;
-        d.big = (i32 *)(mem + o_big[i]);
         d.boff = (i64 *)(mem + o_boff) + (size_t)i * (P + 1);
-        d.spill = (i64 *)(mem + o_sp[i]);
-        d.spill2 = (i64 *)(mem + o_sp2[i]);
-        d.n_spill = cnt + N_SPILL + i;
-        d.n_spill2 = cnt + N_SPILL2 + i;
+        d.best = (unsigned long long *)(mem + o_d[6 * i]);
+        d.active = (i32 *)(mem + o_d[6 * i + 1]);
+        d.big = (i32 *)(mem + o_d[6 * i + 2]);
+        d.spill = (i64 *)(mem + o_d[6 * i + 3]);
+        d.spill2 = (i64 *)(mem + o_d[6 * i + 4]);
+        d.sum = acc + (size_t)p * 6 * P + (size_t)(i & 1) * 2 * P;
+        d.count = acc + (size_t)p * 6 * P + (size_t)(4 + (i & 1)) * P;
+        d.tkey = (u64 *)(mem + o_tkey[p]);
+        d.tval = (i32 *)(mem + o_d[6 * (i & ~1) + 5]);
+        d.tmask = T[p] - 1;
     }
-    u64 *tkey = (u64 *)(mem + o_tkey);
-    i32 *tval = (i32 *)(mem + o_tval);
-    const i64 most = std::max(C[0], C[1]);
-    const dim3 both(grid_of(most), 2);
+    const Scale *ds = (const Scale *)(mem + o_scales);
+    PairArgs a{};
+    a.d = (const Direction *)(mem + o_dirs);
+    a.n = nd;
+    a.P = P;
+    a.tab = tab;
+    a.next_global = cnt + nd * COUNTERS;
     do {
         if ((rc = cuda_status(cudaMemsetAsync(mem, 0, zeroed, st)))) break;
+        if ((rc = cuda_status(cudaMemcpyAsync(mem + o_scales, scales.data(), ns * sizeof(Scale),
+                                              cudaMemcpyHostToDevice, st))))
+            break;
+        if ((rc = cuda_status(cudaMemcpyAsync(mem + o_dirs, dirs.data(), nd * sizeof(Direction),
+                                              cudaMemcpyHostToDevice, st))))
+            break;
+        // node -> communities
+        count_memberships<<<dim3(grid_of(most_m), ns), 256, 0, st>>>(ds); note_launch();
+        i64 *wide = (i64 *)(mem + o_wide), *mptr = (i64 *)(mem + o_mptr);
+        widen_i32<<<grid_of(ns * n), 256, 0, st>>>((const i32 *)(mem + o_mcnt), ns * n, wide); note_launch();
+        if ((rc = scan_exclusive_i64(wide, mptr, ns * n, mptr + ns * n, st))) break;
+        fill_memberships<<<dim3(grid_of(32 * most), ns), 256, 0, st>>>(ds); note_launch();
+        comm_parts<<<dim3(grid_of(most), ns), 256, 0, st>>>(ds, part_off, P, n); note_launch();
         // identical communities
-        hash_insert<<<grid_of(C[1]), 256, 0, st>>>(Y.comm_hash, C[1], tkey, tval, T - 1); note_launch();
-        match_identical<<<grid_of(32 * C[0]), 256, 0, st>>>(X.comm_ptr, X.comm_nodes, X.comm_hash, C[0], Y.comm_ptr,
-                                                            Y.comm_nodes, tkey, tval, T - 1, mem + o_zero[0],
-                                                            mem + o_zero[1]); note_launch();
-        init_best<<<both, 256, 0, st>>>(a); note_launch();
-        list_big<<<both, 256, 0, st>>>(a, 0); note_launch();
-        big_offsets<<<dim3(1, 2), 32, 0, st>>>(a); note_launch();
-        list_big<<<both, 256, 0, st>>>(a, 1); note_launch();
-        pairs_warp<<<(unsigned)std::min<i64>((C[0] + C[1] + NMI_WARPS - 1) / NMI_WARPS, 152 * 5), NMI_WARPS * 32, 0,
+        hash_insert<<<dim3(grid_of(most), np), 256, 0, st>>>(a); note_launch();
+        match_identical<<<dim3(grid_of(32 * most), np), 256, 0, st>>>(a); note_launch();
+        const dim3 each(grid_of(most), nd);
+        init_best<<<each, 256, 0, st>>>(a); note_launch();
+        list_big<<<each, 256, 0, st>>>(a, 0); note_launch();
+        big_offsets<<<dim3(1, nd), 32, 0, st>>>(a); note_launch();
+        list_big<<<each, 256, 0, st>>>(a, 1); note_launch();
+        pairs_warp<<<(unsigned)std::min<i64>((nd * most + NMI_WARPS - 1) / NMI_WARPS, 152 * 5), NMI_WARPS * 32, 0,
                      st>>>(a); note_launch();
         const size_t bsm = 2 * sizeof(i32) * BLK_TABLE + sizeof(unsigned short) * (BLK_TABLE / 2);
         if ((rc = cuda_status(cudaFuncSetAttribute(pairs_block, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    (int)bsm))))
             break;
-        pairs_block<<<(unsigned)std::min<i64>(C[0] + C[1], 152 * 3), BLK_WARPS * 32, bsm, st>>>(a); note_launch();
+        pairs_block<<<(unsigned)std::min<i64>(nd * most, 152 * 3), BLK_WARPS * 32, bsm, st>>>(a); note_launch();
         if (most > BLK_TABLE / 2) {
-            unsigned long long h[2] = {0, 0};
-            if ((rc = cuda_status(cudaMemcpyAsync(h, cnt + N_SPILL2, sizeof(h), cudaMemcpyDeviceToHost, st)))) break;
+            std::vector<unsigned long long> h(nd, 0);
+            if ((rc = cuda_status(cudaMemcpyAsync(h.data(), cnt + N_SPILL2 * nd, nd * 8, cudaMemcpyDeviceToHost, st))))
+                break;
             if ((rc = cuda_status(cudaStreamSynchronize(st)))) break;
-            for (int i = 0; i < 2 && rc == MSCD_OK; ++i)
-                if (h[i]) rc = global_tier(a, i, (i64)h[i], st);
+            for (int i = 0; i < nd && rc == MSCD_OK; ++i)
+                if (h[i]) rc = global_tier(a, i, dirs[i], (i64)h[i], st);
             if (rc) break;
         }
-        normalise_sum<<<both, 256, 0, st>>>(a, acc); note_launch();
+        normalise_sum<<<each, 256, 0, st>>>(a); note_launch();
         rc = cuda_status(cudaGetLastError());
     } while (0);
     cudaFreeAsync(mem, st);
     return rc;
+}
+
+// Scratch of a scale in chunk_terms, about.
+size_t scale_scratch(const ScaleResult &R, i64 n, i64 P) {
+    return (size_t)n * 24 + (size_t)R.n_nodes * 4 + (size_t)R.n_comms * 140 + (size_t)P * 80;
 }
 
 }  // namespace
@@ -870,7 +911,6 @@ int nmi_chain(const ScaleResult *sc, int32_t S, i64 n, const i64 *part_off, int3
     if (pairs == 0 || n <= 0) return MSCD_OK;
     double *tab = nullptr;
     unsigned long long *acc = nullptr;
-    ScaleData data[2];  // of scales s and s + 1, by parity
     const size_t words = 6 * (size_t)P;
     std::vector<unsigned long long> h(words * pairs);
     int rc = MSCD_OK;
@@ -881,12 +921,20 @@ int nmi_chain(const ScaleResult *sc, int32_t S, i64 n, const i64 *part_off, int3
         }
         if ((rc = dev_alloc(&acc, (i64)h.size(), st))) break;
         if ((rc = cuda_status(cudaMemsetAsync(acc, 0, h.size() * sizeof(acc[0]), st)))) break;
-        for (int32_t s = 0; s < S && rc == MSCD_OK; ++s) {
-            free_scale(&data[s & 1], st);
-            if (sc[s].n_comms <= 0) continue;
-            if ((rc = build_scale(sc[s], n, part_off, P, &data[s & 1], st))) break;
-            if (s > 0 && sc[s - 1].n_comms > 0)
-                rc = pair_terms(sc[s - 1], sc[s], data[(s - 1) & 1], data[s & 1], P, tab, acc + words * (s - 1), st);
+        // as many scales at a time as CHUNK_SCRATCH bytes hold (two at least);
+        // a scale without communities ends a run of pairs
+        for (int32_t s0 = 0; s0 + 1 < S && rc == MSCD_OK;) {
+            int32_t s1 = s0;
+            size_t bytes = 0;
+            while (s1 < S && sc[s1].n_comms > 0) {
+                bytes += scale_scratch(sc[s1], n, P);
+                if (s1 - s0 >= 2 && (bytes > CHUNK_SCRATCH || s1 - s0 >= CHUNK_SCALES)) break;
+                ++s1;
+            }
+            if (s1 - s0 >= 2) rc = chunk_terms(sc + s0, s1 - s0, n, part_off, P, tab, acc + words * s0, st);
+            // the last scale of a chunk is the first of the next one
+            s0 = s1 < S && sc[s1].n_comms <= 0 ? s1 + 1 : std::max(s1 - 1, s0 + 1);
+            if (s1 == S) break;
         }
         if (rc) break;
         if ((rc = cuda_status(cudaMemcpyAsync(h.data(), acc, h.size() * sizeof(acc[0]), cudaMemcpyDeviceToHost, st))))
@@ -902,7 +950,6 @@ int nmi_chain(const ScaleResult *sc, int32_t S, i64 n, const i64 *part_off, int3
                 nmi[(size_t)s * P + p] = 1.0 - 0.5 * (sx / (double)cx + sy / (double)cy);
             }
     } while (0);
-    for (auto &x : data) free_scale(&x, st);
     cudaFreeAsync(tab, st);
     cudaFreeAsync(acc, st);
     if (rc) cudaStreamSynchronize(st);
