@@ -12,18 +12,18 @@ size_t grow_bytes_i32(int cap, bool smem);
 
 namespace {
 
-// Exact 64-bit sums for weighted graphs, else 16-bit d_in and degree when
+// Exact 64-bit sums for weighted graphs, else 15-bit d_in and degree when
 // every degree fits, 32-bit beyond.
 int dispatch(const GrowArgs &a, int blocks, int threads, size_t smem, cudaStream_t st, int *occ) {
     if (a.G.wfx) return grow_launch_weighted(a, blocks, threads, smem, st, occ);
-    return (a.G.kmax < 65536 ? grow_launch_u16 : grow_launch_i32)(a, blocks, threads, smem, st, occ);
+    return (a.G.kmax < 32768 ? grow_launch_u16 : grow_launch_i32)(a, blocks, threads, smem, st, occ);
 }
 
 }  // namespace
 
 size_t grow_state_bytes(const DevGraph &G, int cap, bool smem) {
     if (G.wfx) return grow_bytes_weighted(cap, smem);
-    return G.kmax < 65536 ? grow_bytes_u16(cap, smem) : grow_bytes_i32(cap, smem);
+    return G.kmax < 32768 ? grow_bytes_u16(cap, smem) : grow_bytes_i32(cap, smem);
 }
 
 int grow_launch(const GrowArgs &a, int blocks, int threads, size_t smem, cudaStream_t st) {

@@ -30,7 +30,7 @@
 // Ranking keys are binary32 log2 d - alpha log2 k, compared with a certified
 // bound; pairs closer than the bound are ordered by the exact comparator.
 // With u = 2^-24 and L = log2 of the largest degree, a key carries at most
-// 1.5u (conversion of d) + 4u (1+L) (__log2f: 2 ulp, or 2^-22 absolute on
+// 1.5u (conversion of d) + 4u (1+L) (lg2.approx: 2 ulp, or 2^-22 absolute on
 // [1/2, 2]) + 5u alpha (1+L) (the stored log2 k, fl(alpha), product) +
 // u (1+alpha) L (difference) <= 7u (1+alpha)(1+L) of error;
 // E = 2^-20 (1+alpha)(1+L) = 16u (1+alpha)(1+L) per key is above it.
@@ -47,8 +47,8 @@
 // of log2 d - log2 k (it shares both logarithms with the key), lets the bulk
 // test skip the groups whose nodes cannot pass.
 //
-// State per warp: node slots (d_in, key, id with the member flag in its sign
-// bit; k_u is read from the graph's degree array, which every unit shares),
+// State per warp: node slots (see Slots; the id has the member flag in its sign
+// bit),
 // a member list (slots in joining order, for the prune passes and the
 // output), group bounds and an open-addressing hash node -> slot, in shared memory
 // (first class) or in a global-memory arena (larger classes, run at high
@@ -69,8 +69,8 @@
 // in shared memory: with all of it inlined the kernel wanted 160 registers,
 // spilled in the loop at 16 units per SM and waited for instructions.  Growth
 // of the 1-of-8 run of the 100,000-node graph (250,000 units, the shared class
-// and the 8,192-slot one): 48 + 237 ms before, 30 + 156 now; of the 1-of-80 run
-// of the weighted 1M-node graph 41 + 461, now 30 + 283.
+// and the 8,192-slot one): 48 + 237 ms before, 28 + 151 now; of the 1-of-80 run
+// of the weighted 1M-node graph 41 + 461, now 29 + 280.
 #pragma once
 
 #include <type_traits>
@@ -82,6 +82,7 @@
 namespace {
 
 // A slot's id holds the node id (< 2^31) with the member flag in bit 31.
+typedef unsigned short u16;
 constexpr i32 MEMBER_BIT = (i32)0x80000000u;
 __device__ __forceinline__ i32 node_of(i32 x) { return x & 0x7fffffff; }
 constexpr int HASH_MIN = 256;  // buckets of a unit's table at its start
@@ -95,11 +96,27 @@ __device__ __forceinline__ float unord(int o) { return __int_as_float(o >= 0 ? o
 constexpr int ORD_NEG_INF = (int)(0xff800000u ^ 0x7fffffffu);
 constexpr float NEG_INF = -__builtin_huge_valf();
 
+// __log2f for arguments that are 0 or at least 1 (the same value: only
+// denormal arguments differ, which that handles with three more instructions).
+__device__ __forceinline__ float log2_int(float x) {
+    float y;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// An integer below 2^23 as binary32, without the conversion unit (it shares
+// its quarter rate with the logarithm).
+__device__ __forceinline__ float small2f(u32 x) { return __uint_as_float(0x4b000000u | x) - 0x1p23f; }
+
+__device__ __forceinline__ float d2f(i64 d) { return __ll2float_rn(d); }
+__device__ __forceinline__ float d2f(i32 d) { return __int2float_rn(d); }
+
 // Node slots.  Weighted: one 16-byte record, a single sector per visit; the
 // node's degree and its logarithm are read from the graph's arrays.
-// Unweighted: id and key in 8 bytes, d_in and the degree (2 or 4 bytes each)
-// apart, so that scans of the slots (argmax, bulk rejection, prune) and visits
-// of nodes already met read nothing of the graph but the row.
+// Unweighted: the degree is in the slot, so that scans of the slots (argmax,
+// bulk rejection, prune) and visits of nodes already met read nothing of the
+// graph but the row; degrees from 32,768 on have id and key in 8 bytes, d_in and
+// the degree in 8 bytes apart.
 struct __align__(16) WeightedSlot {
     i64 d;
     i32 id;
@@ -126,7 +143,7 @@ struct Slots {  // unweighted
         d = (D)x.d;
         k = (D)x.k;
     }
-    __device__ __forceinline__ void get(int s, i32 &id, float &key, D &d, D &k) const {
+    __device__ __forceinline__ void get(int s, i32 &id, float &key, D &d, D &k, float) const {
         const DK x = dk[s];
         const int2 y = ik[s];
         id = y.x;
@@ -134,12 +151,13 @@ struct Slots {  // unweighted
         d = (D)x.d;
         k = (D)x.k;
     }
+    __device__ __forceinline__ static float log_d(D d) { return log2_int(d2f(d)); }
     __device__ __forceinline__ static i64 degree(const DevGraph &, i32, D k) { return (i64)k; }
     __device__ __forceinline__ static float log_degree(const DevGraph &, i32, D k) {
-        return __log2f(__int2float_rn(k));
+        return log2_int(d2f(k));
     }
     __device__ __forceinline__ i32 id(int s) const { return ik[s].x; }
-    __device__ __forceinline__ float key(int s) const { return __int_as_float(ik[s].y); }
+    __device__ __forceinline__ float key(int s, float) const { return __int_as_float(ik[s].y); }
     __device__ __forceinline__ void put_new(int s, i32 id, float key, D d, D k) const {
         DK x;
         x.d = (VT)d;
@@ -151,10 +169,71 @@ struct Slots {  // unweighted
         ik[s].y = __float_as_int(key);
         dk[s].d = (VT)d;
     }
-    __device__ __forceinline__ void put(int s, i32 id, float key) const { ik[s] = make_int2(id, __float_as_int(key)); }
+    __device__ __forceinline__ void put_member(int s, i32 id, D, D) const {
+        ik[s] = make_int2(id | MEMBER_BIT, __float_as_int(NEG_INF));
+    }
     __device__ __forceinline__ void put_id(int s, i32 id) const { ik[s].x = id; }
-    __device__ __forceinline__ void put_key(int s, float key) const { ik[s].y = __float_as_int(key); }
+    __device__ __forceinline__ void put_key(int s, float key, D) const { ik[s].y = __float_as_int(key); }
     __device__ __forceinline__ void put_d(int s, D d) const { dk[s].d = (VT)d; }
+};
+
+// Degrees below 32,768 (15 bits): id, d_in and degree in 8 bytes, and in place of
+// the key a flag in d_in's top bit for a node outside the queue.  The key is a
+// function of d_in and the degree, two logarithms away, which the scans of a few
+// groups can afford; a visit is one sector and a 2-byte store, and 15 states
+// instead of 12 fit an SM's shared memory.  Against keys in the slots (12 bytes):
+// the shared class of the 10,000-node run 27.7 -> 23.9 ms, of the 1,000-node run
+// 1.69 -> 1.37, the 8,192-slot class of the union of 12 graphs 208 -> 193, of the
+// 1-of-8 run of the 100,000-node graph 156 -> 151.
+template <>
+struct Slots<u16, false> {
+    typedef i32 D;
+    static constexpr size_t BYTES = 8;
+    static constexpr u32 OUT = 0x8000u;
+    struct __align__(8) Rec {
+        i32 id;
+        u16 d, k;
+    };
+    Rec *r;
+    __device__ __forceinline__ void at(unsigned char *base, int) { r = (Rec *)base; }
+    __device__ __forceinline__ void get(int s, i32 &id, D &d, D &k) const {
+        const int2 x = *(const int2 *)&r[s];
+        id = x.x;
+        d = x.y & 0x7fff;
+        k = (D)((u32)x.y >> 16);
+    }
+    __device__ __forceinline__ static float key_of(int y, float alpha32) {
+        return (u32)y & OUT ? NEG_INF
+                            : fmaf(-alpha32, log2_int(small2f((u32)y >> 16)), log2_int(small2f((u32)y & 0x7fffu)));
+    }
+    __device__ __forceinline__ void get(int s, i32 &id, float &key, D &d, D &k, float alpha32) const {
+        const int2 x = *(const int2 *)&r[s];
+        id = x.x;
+        d = x.y & 0x7fff;
+        k = (D)((u32)x.y >> 16);
+        key = key_of(x.y, alpha32);
+    }
+    __device__ __forceinline__ static float log_d(D d) { return log2_int(small2f((u32)d)); }
+    __device__ __forceinline__ static i64 degree(const DevGraph &, i32, D k) { return (i64)k; }
+    __device__ __forceinline__ static float log_degree(const DevGraph &, i32, D k) {
+        return log2_int(small2f((u32)k));
+    }
+    __device__ __forceinline__ i32 id(int s) const { return r[s].id; }
+    __device__ __forceinline__ float key(int s, float alpha32) const {
+        return key_of(((const int2 *)r)[s].y, alpha32);
+    }
+    __device__ __forceinline__ static u16 flagged(float key, D d) { return (u16)(key == NEG_INF ? (u32)d | OUT : (u32)d); }
+    __device__ __forceinline__ void put_new(int s, i32 id, float key, D d, D k) const {
+        *(int2 *)&r[s] = make_int2(id, (int)((u32)flagged(key, d) | ((u32)k << 16)));
+    }
+    __device__ __forceinline__ void put(int s, i32, float, D d) const { r[s].d = (u16)d; }
+    __device__ __forceinline__ void put_member(int s, i32 id, D d, D k) const {
+        *(int2 *)&r[s] = make_int2(id | MEMBER_BIT, (int)((u32)d | OUT | ((u32)k << 16)));
+    }
+    __device__ __forceinline__ void put_id(int s, i32 id) const { r[s].id = id; }
+    __device__ __forceinline__ void put_key(int s, float key, D d) const { r[s].d = flagged(key, d); }
+    // of a member, or where no queue is kept
+    __device__ __forceinline__ void put_d(int s, D d) const { r[s].d = (u16)((u32)d | OUT); }
 };
 
 template <>
@@ -163,7 +242,7 @@ struct Slots<i64, true> {
     static constexpr size_t BYTES = 16;
     WeightedSlot *r;
     __device__ __forceinline__ void at(unsigned char *base, int) { r = (WeightedSlot *)base; }
-    __device__ __forceinline__ void get(int s, i32 &id, float &key, D &d, D &k) const {
+    __device__ __forceinline__ void get(int s, i32 &id, float &key, D &d, D &k, float) const {
         const int4 x = *(const int4 *)&r[s];
         d = (i64)((u64)(u32)x.x | ((u64)(u32)x.y << 32));
         id = x.z;
@@ -172,33 +251,30 @@ struct Slots<i64, true> {
     }
     __device__ __forceinline__ void get(int s, i32 &id, D &d, D &k) const {
         float key;
-        get(s, id, key, d, k);
+        get(s, id, key, d, k, 0.0f);
     }
+    __device__ __forceinline__ static float log_d(D d) { return log2_int(d2f(d)); }
     __device__ __forceinline__ static i64 degree(const DevGraph &G, i32 id, D) { return G.k[id]; }
     __device__ __forceinline__ static float log_degree(const DevGraph &G, i32 id, D) { return G.logk[id]; }
     __device__ __forceinline__ i32 id(int s) const { return r[s].id; }
-    __device__ __forceinline__ float key(int s) const { return r[s].key; }
+    __device__ __forceinline__ float key(int s, float) const { return r[s].key; }
     __device__ __forceinline__ void put(int s, i32 id, float key, D d) const {
         *(int4 *)&r[s] = make_int4((int)(u32)(u64)d, (int)(u32)((u64)d >> 32), id, __float_as_int(key));
     }
     __device__ __forceinline__ void put_new(int s, i32 id, float key, D d, D) const { put(s, id, key, d); }
-    __device__ __forceinline__ void put(int s, i32 id, float key) const {
-        *(int2 *)&r[s].id = make_int2(id, __float_as_int(key));
+    __device__ __forceinline__ void put_member(int s, i32 id, D, D) const {
+        *(int2 *)&r[s].id = make_int2(id | MEMBER_BIT, __float_as_int(NEG_INF));
     }
     __device__ __forceinline__ void put_id(int s, i32 id) const { r[s].id = id; }
-    __device__ __forceinline__ void put_key(int s, float key) const { r[s].key = key; }
+    __device__ __forceinline__ void put_key(int s, float key, D) const { r[s].key = key; }
     __device__ __forceinline__ void put_d(int s, D d) const { r[s].d = d; }
 };
-
-__device__ __forceinline__ float d2f(i64 d) { return __ll2float_rn(d); }
-__device__ __forceinline__ float d2f(i32 d) { return __int2float_rn(d); }
 
 // Hash buckets: 0 is empty, else the slot + 1 and what tells most other nodes
 // apart without reading their slots (in the arena a slot is a memory round
 // trip; a bucket's neighbour is in the same sector).  16 bits: the slot alone
 // (shared memory); 32 bits: slot and 16 bits of the hash (up to 32768 slots);
 // 64 bits: slot and node id.
-typedef unsigned short u16;
 __device__ __forceinline__ u32 hash_node(i32 v) { return (u32)v * 0x9E3779B1u; }
 template <class BT>
 __device__ __forceinline__ BT bucket(int slot, i32 v) {
@@ -246,6 +322,7 @@ struct State {
     __device__ __forceinline__ static float log_degree(const DevGraph &G, i32 id, D k) {
         return Slots<VT, WEIGHTED>::log_degree(G, id, k);
     }
+    __device__ __forceinline__ static float log_d(D d) { return Slots<VT, WEIGHTED>::log_d(d); }
 };
 
 // Layout: slots | hash | member list | group bounds.  Rounded up to
@@ -469,9 +546,9 @@ __device__ __forceinline__ int max_bound(const ST &st, int G) {
 
 // This lane's node of group gg (slot -1: none queued; no group: gg < 0).
 template <class ST>
-__device__ __forceinline__ Pick<typename ST::D> queued_of(const ST &st, int ns, int gg) {
+__device__ __forceinline__ Pick<typename ST::D> queued_of(const ST &st, int ns, int gg, float alpha32) {
     Pick<typename ST::D> p = {gg * 32 + (int)(threadIdx.x & 31), 0, NEG_INF, 0, 0};
-    if ((u32)p.slot < (u32)ns) st.sl.get(p.slot, p.id, p.key, p.d, p.k);
+    if ((u32)p.slot < (u32)ns) st.sl.get(p.slot, p.id, p.key, p.d, p.k, alpha32);
     if (p.key == NEG_INF) p.slot = -1;
     return p;
 }
@@ -499,7 +576,7 @@ __device__ __forceinline__ Pick<typename ST::D> queue_top(const ST &st, const Li
 #pragma unroll 1
             for (; ball; ball &= ball - 1) {
                 last = base + __ffs(ball) - 1;
-                const Pick<D> p = queued_of(st, U.ns, last);
+                const Pick<D> p = queued_of(st, U.ns, last, U.alpha32);
                 gkey = p.key;
                 // the group's exact bound; candidates stay lane-local until the end
                 const int o = __reduce_max_sync(FULL_MASK, ord(gkey));
@@ -524,7 +601,7 @@ __device__ __forceinline__ Pick<typename ST::D> queue_top(const ST &st, const Li
     t = warp_best<ST>(t, U.E2);
     if (t.slot >= 0 && t.slot >> 5 != last) {
         const int i = (t.slot & ~31) + lane;
-        gkey = i < U.ns ? st.sl.key(i) : NEG_INF;
+        gkey = i < U.ns ? st.sl.key(i, U.alpha32) : NEG_INF;
     }
     return t;
 }
@@ -656,7 +733,7 @@ __device__ __forceinline__ bool expand(const ST &st, const GrowArgs &a, Live &U,
             if (ST::WEIGHTED) d += sign < 0 ? -w : w;
             else d += sign;
             if (requeue && !member) {
-                const float ld = __log2f(d2f(d));
+                const float ld = ST::log_d(d);
                 if (!ST::WEIGHTED) lk = ST::log_degree(a.G, v, k);
                 const float key = fmaf(-U.alpha32, lk, ld);
                 if (need) st.sl.put_new(s, v, key, d, k);
@@ -722,11 +799,11 @@ __device__ __forceinline__ bool build_queue(const ST &st, const Unit &U) {
             const int i = (g0 + j) * 32 + lane;
             float key = NEG_INF, q = NEG_INF;
             if (id[j] >= 0 && d[j] > 0) {
-                const float ld = __log2f(d2f(d[j]));
+                const float ld = ST::log_d(d[j]);
                 key = fmaf(-alpha32, lk[j], ld);
                 q = ld - lk[j];
             }
-            if (i < ns) st.sl.put_key(i, key);
+            if (i < ns) st.sl.put_key(i, key, d[j]);
             const int o = __reduce_max_sync(FULL_MASK, ord(key));
             const int qo = __reduce_max_sync(FULL_MASK, ord(q));
             best = max(best, qo);
@@ -768,7 +845,7 @@ __device__ __forceinline__ Pick<typename ST::D> best_passing(const ST &st, Unit 
             for (int j = 0; j < GROUPS; ++j) {
                 gg[j] = ball ? base + __ffs(ball) - 1 : -1;
                 ball &= ball - 1;
-                p[j] = queued_of(st, ns, gg[j]);
+                p[j] = queued_of(st, ns, gg[j], alpha32);
             }
 #pragma unroll
             for (int j = 0; j < GROUPS; ++j) kd[j] = p[j].slot >= 0 ? ST::degree(args().G, p[j].id, p[j].k) : 1;
@@ -779,7 +856,7 @@ __device__ __forceinline__ Pick<typename ST::D> best_passing(const ST &st, Unit 
                 const float df = d2f(p[j].d), kf = exact::i2f(kd[j]);
                 // the group's d/k bound made exact again (members and rejected
                 // nodes have left the queue since it was last raised)
-                const int qo = __reduce_max_sync(FULL_MASK, queued ? ord(__log2f(df) - __log2f(kf)) : ORD_NEG_INF);
+                const int qo = __reduce_max_sync(FULL_MASK, queued ? ord(log2_int(df) - log2_int(kf)) : ORD_NEG_INF);
                 if (lane == 0) st.qmax[gg[j]] = qo;
                 if (!queued || exact::lowers(Kf, Vf, df, kf, alpha32)) continue;
                 u32 fl = 0;
@@ -810,9 +887,9 @@ __device__ __forceinline__ void drop_before(const ST &st, const Pick<typename ST
         while (ball) {
             const int gg = base + __ffs(ball) - 1;
             ball &= ball - 1;
-            const Pick<typename ST::D> p = queued_of(st, ns, gg);
+            const Pick<typename ST::D> p = queued_of(st, ns, gg, U.alpha32);
             const bool drop = p.slot >= 0 && p.slot != t.slot && ranks_before<ST>(p, t, E2);
-            if (drop) st.sl.put_key(p.slot, NEG_INF);
+            if (drop) st.sl.put_key(p.slot, NEG_INF, p.d);
             // the group's key bound made exact again
             const int o = __reduce_max_sync(FULL_MASK, drop ? ORD_NEG_INF : ord(p.key));
             if (lane == 0) st.gmax[gg] = o;
@@ -1012,6 +1089,7 @@ __device__ __noinline__ int next_row(int why) {
                 add = t.slot;
                 u = t.id;
                 d = t.d;
+                k = t.k;
             }
             // none passes: every queued node is popped and rejected, the grow
             // pass ends (the next round rebuilds every key)
@@ -1076,7 +1154,7 @@ __device__ __noinline__ int next_row(int why) {
     }
     __syncwarp();
     if (lane == 0) {
-        st.sl.put(add, u | MEMBER_BIT, NEG_INF);
+        st.sl.put_member(add, u, d, k);
         st.mem[U.nm] = (typename ST::MT)add;
         U.nm++;
         U.K += 2 * (i64)d;
@@ -1300,7 +1378,7 @@ __device__ __forceinline__ void grow_unit(const ST &st, const GrowArgs &a, i64 u
             __syncwarp();
             if (lane == 0) {
                 st.gmax[top.slot >> 5] = o;
-                st.sl.put(top.slot, top.id | MEMBER_BIT, NEG_INF);
+                st.sl.put_member(top.slot, top.id, top.d, top.k);
                 st.mem[U.nm] = (typename ST::MT)top.slot;
                 S.adds += 1ull;
                 S.added = true;
