@@ -313,20 +313,21 @@ __device__ __forceinline__ bool remove_test(i64 K, i64 V, i64 d, i64 k, double a
 //   x(6+3x)/(6+6x+x^2) <= log1p(x) <= x(6+x)/(6+4x),   the same for y
 // (Pade approximants; the differences have derivatives of one sign for
 // positive arguments: x^4/((1+x)(6+6x+x^2)^2) and 4x^3/((1+x)(6+4x)^2)).
-// Each side is computed within 20 roundings of 2^-24 (the fast division within
-// 2 ulp); the margin 2^-18 covers both.
-__device__ __forceinline__ float log1p_low(float x) {
-    return __fdividef(x * fmaf(3.0f, x, 6.0f), fmaf(x, x + 6.0f, 6.0f));
-}
-__device__ __forceinline__ float log1p_high(float x) { return __fdividef(x * (6.0f + x), fmaf(4.0f, x, 6.0f)); }
-
-// (K+2d)/(V+k)^alpha > K/V^alpha for certain.
-__device__ __forceinline__ bool raises(float K, float V, float d, float k, float alpha32) {
-    return log1p_low(__fdividef(2.0f * d, K)) > alpha32 * log1p_high(__fdividef(k, V)) * (1.0f + 0x1p-18f);
+// Multiplied out, each side is a product of sums of positive terms, computed
+// within 40 roundings of 2^-24 (the fast division counts as 4, a quotient may
+// enter squared); the margin 2^-17 covers both.  A side that overflows is the
+// larger one: its remaining factors are above 1.  No divisions here, so that
+// scans over many nodes only multiply (by 2/K and 1/V).
+//
+// (K+2d)/(V+k)^alpha > K/V^alpha for certain, x = 2d/K, y = k/V.
+__device__ __forceinline__ bool raises(float x, float y, float alpha32) {
+    return x * fmaf(3.0f, x, 6.0f) * fmaf(4.0f, y, 6.0f) >
+           alpha32 * y * (6.0f + y) * fmaf(x, x + 6.0f, 6.0f) * (1.0f + 0x1p-17f);
 }
 // (K+2d)/(V+k)^alpha < K/V^alpha for certain.
-__device__ __forceinline__ bool lowers(float K, float V, float d, float k, float alpha32) {
-    return log1p_high(__fdividef(2.0f * d, K)) < alpha32 * log1p_low(__fdividef(k, V)) * (1.0f - 0x1p-18f);
+__device__ __forceinline__ bool lowers(float x, float y, float alpha32) {
+    return x * (6.0f + x) * fmaf(y, y + 6.0f, 6.0f) <
+           alpha32 * y * fmaf(3.0f, y, 6.0f) * fmaf(4.0f, x, 6.0f) * (1.0f - 0x1p-17f);
 }
 
 }  // namespace exact

@@ -151,6 +151,7 @@ struct Slots {  // unweighted
         d = (D)x.d;
         k = (D)x.k;
     }
+    __device__ __forceinline__ static float to_float(D x) { return d2f(x); }
     __device__ __forceinline__ static float log_d(D d) { return log2_int(d2f(d)); }
     __device__ __forceinline__ static i64 degree(const DevGraph &, i32, D k) { return (i64)k; }
     __device__ __forceinline__ static float log_degree(const DevGraph &, i32, D k) {
@@ -213,6 +214,7 @@ struct Slots<u16, false> {
         k = (D)((u32)x.y >> 16);
         key = key_of(x.y, alpha32);
     }
+    __device__ __forceinline__ static float to_float(D x) { return small2f((u32)x); }
     __device__ __forceinline__ static float log_d(D d) { return log2_int(small2f((u32)d)); }
     __device__ __forceinline__ static i64 degree(const DevGraph &, i32, D k) { return (i64)k; }
     __device__ __forceinline__ static float log_degree(const DevGraph &, i32, D k) {
@@ -253,6 +255,7 @@ struct Slots<i64, true> {
         float key;
         get(s, id, key, d, k, 0.0f);
     }
+    __device__ __forceinline__ static float to_float(D x) { return d2f(x); }
     __device__ __forceinline__ static float log_d(D d) { return log2_int(d2f(d)); }
     __device__ __forceinline__ static i64 degree(const DevGraph &G, i32 id, D) { return G.k[id]; }
     __device__ __forceinline__ static float log_degree(const DevGraph &G, i32 id, D) { return G.logk[id]; }
@@ -323,6 +326,11 @@ struct State {
         return Slots<VT, WEIGHTED>::log_degree(G, id, k);
     }
     __device__ __forceinline__ static float log_d(D d) { return Slots<VT, WEIGHTED>::log_d(d); }
+    __device__ __forceinline__ static float d_float(D d) { return Slots<VT, WEIGHTED>::to_float(d); }
+    // the degree of a slot's node as binary32 (unweighted: k is in the slot)
+    __device__ __forceinline__ static float k_float(const DevGraph &G, i32 id, D k) {
+        return WEIGHTED ? exact::i2f(G.k[id]) : Slots<VT, WEIGHTED>::to_float(k);
+    }
 };
 
 // Layout: slots | hash | member list | group bounds.  Rounded up to
@@ -830,7 +838,8 @@ __device__ __forceinline__ Pick<typename ST::D> best_passing(const ST &st, Unit 
     const int lane = threadIdx.x & 31, ns = U.ns;
     const int G = (ns + 31) >> 5;
     const int othr = pass_bound(U, args().G.kmax);
-    const float Kf = exact::i2f(U.K), Vf = exact::i2f(U.V), alpha32 = U.alpha32, E2 = U.E2;
+    const float x_d = __fdividef(2.0f, exact::i2f(U.K)), y_k = __fdividef(1.0f, exact::i2f(U.V));
+    const float alpha32 = U.alpha32, E2 = U.E2;
     Pick<D> t = {-1, 0, NEG_INF, 0, 0};
 #pragma unroll 1
     for (int base = 0; base < G; base += 32) {
@@ -840,7 +849,7 @@ __device__ __forceinline__ Pick<typename ST::D> best_passing(const ST &st, Unit 
         while (ball) {
             int gg[GROUPS];
             Pick<D> p[GROUPS];
-            i64 kd[GROUPS];
+            float kf[GROUPS];
 #pragma unroll
             for (int j = 0; j < GROUPS; ++j) {
                 gg[j] = ball ? base + __ffs(ball) - 1 : -1;
@@ -848,20 +857,21 @@ __device__ __forceinline__ Pick<typename ST::D> best_passing(const ST &st, Unit 
                 p[j] = queued_of(st, ns, gg[j], alpha32);
             }
 #pragma unroll
-            for (int j = 0; j < GROUPS; ++j) kd[j] = p[j].slot >= 0 ? ST::degree(args().G, p[j].id, p[j].k) : 1;
+            for (int j = 0; j < GROUPS; ++j) kf[j] = p[j].slot >= 0 ? ST::k_float(args().G, p[j].id, p[j].k) : 1.0f;
 #pragma unroll
             for (int j = 0; j < GROUPS; ++j) {
                 if (gg[j] < 0) break;
                 const bool queued = p[j].slot >= 0;
-                const float df = d2f(p[j].d), kf = exact::i2f(kd[j]);
+                const float df = ST::d_float(p[j].d), x = df * x_d, y = kf[j] * y_k;
                 // the group's d/k bound made exact again (members and rejected
                 // nodes have left the queue since it was last raised)
-                const int qo = __reduce_max_sync(FULL_MASK, queued ? ord(log2_int(df) - log2_int(kf)) : ORD_NEG_INF);
+                const int qo = __reduce_max_sync(FULL_MASK, queued ? ord(log2_int(df) - log2_int(kf[j])) : ORD_NEG_INF);
                 if (lane == 0) st.qmax[gg[j]] = qo;
-                if (!queued || exact::lowers(Kf, Vf, df, kf, alpha32)) continue;
+                if (!queued || exact::lowers(x, y, alpha32)) continue;
                 u32 fl = 0;
-                const bool pass = exact::raises(Kf, Vf, df, kf, alpha32) ||
-                                  exact::add_test(U.K, U.V, (i64)p[j].d, kd[j], U.alpha, fl);
+                const bool pass = exact::raises(x, y, alpha32) ||
+                                  exact::add_test(U.K, U.V, (i64)p[j].d, ST::degree(args().G, p[j].id, p[j].k),
+                                                  U.alpha, fl);
                 if (fl) atomicOr(&U.xflags, fl);
                 if (pass && (t.slot < 0 || ranks_before<ST>(p[j], t, E2))) t = p[j];
             }
@@ -932,7 +942,9 @@ __device__ __forceinline__ int first_removable(const ST &st, Unit &U, i32 last) 
             if (u == seed || u <= last || u >= bid) continue;
             const i64 Kn = K - 2 * (i64)d[j], Vn = V - kd[j];
             if (Kn <= 0) continue;  // f of the rest is 0
-            if (exact::raises(exact::i2f(Kn), exact::i2f(Vn), d2f(d[j]), exact::i2f(kd[j]), U.alpha32)) continue;
+            if (exact::raises(__fdividef(2.0f * ST::d_float(d[j]), exact::i2f(Kn)),
+                              __fdividef(exact::i2f(kd[j]), exact::i2f(Vn)), U.alpha32))
+                continue;
             u32 fl = 0;
             const bool out = exact::remove_test(K, V, (i64)d[j], kd[j], U.alpha, fl);
             if (fl) atomicOr(&U.xflags, fl);
@@ -1360,10 +1372,11 @@ __device__ __forceinline__ void grow_unit(const ST &st, const GrowArgs &a, i64 u
             // loaded during the test, for the likely addition: the first entries of its row
             load_entries<ST>(G, rs, re, v, w);
             if (U.K != 0) {
-                const float Kf = exact::i2f(U.K), Vf = exact::i2f(U.V), df = d2f(top.d), kf = exact::i2f(k);
-                if (!exact::raises(Kf, Vf, df, kf, U.alpha32)) {
+                const float x = __fdividef(2.0f * ST::d_float(top.d), exact::i2f(U.K));
+                const float y = __fdividef(ST::WEIGHTED ? exact::i2f(k) : ST::d_float(top.k), exact::i2f(U.V));
+                if (!exact::raises(x, y, U.alpha32)) {
                     u32 fl = 0;
-                    const bool pass = !exact::lowers(Kf, Vf, df, kf, U.alpha32) &&
+                    const bool pass = !exact::lowers(x, y, U.alpha32) &&
                                       exact::add_test(U.K, U.V, (i64)top.d, k, S.alpha, fl);
                     if (fl && lane == 0) S.xflags |= fl;
                     if (!pass) {
