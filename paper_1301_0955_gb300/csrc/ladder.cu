@@ -124,8 +124,15 @@ int grow_units(GrowPipe &w, const GrowArgs &proto, i64 n_units, const std::vecto
     while (!tasks.empty() && rc == MSCD_OK) {
         Task t = std::move(tasks.front());
         tasks.erase(tasks.begin());
-        const int cap = ladder[t.cls];
         const i64 n_work = t.all ? n_units : (i64)t.units.size();
+        // A list that is resident all at once takes as long as its longest unit,
+        // and a unit that outgrows its class starts again: such a list goes
+        // straight to the largest class of the same kind (4-byte buckets, bounds
+        // in shared memory).  Lists of at most one unit an SM run in shared
+        // memory, where the smaller class fits.
+        if (!plain && t.cls > 0 && n_work > w.sm_count && n_work <= (i64)w.sm_count * w.p.global_warps_per_sm)
+            while (!in_smem[t.cls] && t.cls + 1 < (int)ladder.size() && ladder[t.cls + 1] <= MIDDLE_SLOTS) ++t.cls;
+        const int cap = ladder[t.cls];
         // A few left-over units (at most one an SM) run in shared memory where a
         // state of their class fits it: there is nothing to hide an arena's
         // latency behind, and the launch lasts as long as its longest unit.
