@@ -10,6 +10,8 @@
 // 1-of-80 weighted 1M-node run the 8,192-slot class takes 283 ms, 316 at 16
 // units (128 registers), 278 at 32 (64, spilling a little; slower than 24
 // where few units run).  The few units of the wider classes take 128.
+#define GROW_CTA_SMEM (size_t)6144  // a CTA's static shared memory and what the system takes, at most
+#define GROW_SM_SMEM (size_t)(228 * 1024)
 #define GLOBAL_CTA_THREADS 128
 #define GLOBAL_MIN_BLOCKS 6
 #define WIDE_MIN_BLOCKS 4

@@ -383,7 +383,8 @@ extern __shared__ __align__(16) unsigned char g_smem[];
 
 // This warp's state: dynamic shared memory (warp w of the CTA at
 // w * state_bytes) or the global arena (warp at its global index), there with
-// the group bounds in shared memory up to 32,768 slots.
+// the group bounds in shared memory up to 32,768 slots, and beyond where the
+// launch has room for them (smem_per_warp; see grow_units).
 template <class ST>
 __device__ __forceinline__ ST my_state(const GrowArgs &a) {
     ST st;
@@ -397,7 +398,7 @@ __device__ __forceinline__ ST my_state(const GrowArgs &a) {
     o += 2 * sizeof(typename ST::BT) * (size_t)C;
     st.mem = (typename ST::MT *)(base + o);
     o += sizeof(typename ST::MT) * (size_t)C;
-    if (ST::SMEM || sizeof(typename ST::BT) == 8) {
+    if (ST::SMEM || (sizeof(typename ST::BT) == 8 && a.smem_per_warp == 0)) {
         st.gmax = (int *)(base + o);
     } else {
         unsigned char *wsm = g_smem + (u32)wib * (u32)a.smem_per_warp;
@@ -546,8 +547,9 @@ struct Live {
 
 template <class ST>
 __device__ __forceinline__ int max_bound(const ST &st, int G) {
+    constexpr int IN_FLIGHT = sizeof(typename ST::BT) == 8 ? 4 : 1;  // thousands of groups, or registers to save
     int m = ORD_NEG_INF;
-#pragma unroll 1
+#pragma unroll IN_FLIGHT
     for (int g = threadIdx.x & 31; g < G; g += 32) m = max(m, st.gmax[g]);
     return __reduce_max_sync(FULL_MASK, m);
 }
@@ -1459,7 +1461,7 @@ __global__ void __launch_bounds__(MAXT, MINB) grow_kernel(const __grid_constant_
 template <class ST, int MAXT, int MINB>
 int launch_k(const GrowArgs &a, int blocks, int threads, size_t smem, cudaStream_t st, int *occ) {
     auto k = grow_kernel<ST, MAXT, MINB>;
-    if (ST::SMEM) {
+    if (ST::SMEM || sizeof(typename ST::BT) == 8) {
         // always the same limit: launches of other sizes may be on their way from other threads
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, GROW_SMEM_MAX);
         if (e != cudaSuccess) return cuda_status(e);

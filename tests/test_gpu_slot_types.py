@@ -50,3 +50,25 @@ def test_hub_degree_and_classes(orc, ctx, h):
     assert (16384 in caps) == (h >= 12000)
     assert any(c > 16384 for c in caps) == (h > 16384)
     ctx.free_graph(gid)
+
+
+@pytest.mark.parametrize("h", [60000, 530000])
+def test_wide_classes(orc, ctx, h):
+    """Group bounds of the wide classes: in shared memory (65,536 slots), in the
+    arena (1,048,576 slots: a unit's bounds exceed an SM's shared memory).  The
+    initial community holds all nodes but two."""
+    n, rp, col, _ = hub_graph(h)
+    G = orc.Graph(n, rp, col)
+    seeds = np.array([0], np.int32)
+    nodes = np.arange(1, h - 1, dtype=np.int32)
+    ptr = np.array([0, nodes.size], np.int64)
+    alphas = np.array([1.0])
+    rc, optr, onodes, of, ost = orc.run(G, alphas, seeds, threads=8, init=(ptr, nodes))
+    assert rc == 0
+    gid = ctx.load_csr(n, rp, col)
+    assert ctx.run_init(gid, alphas, seeds, ptr, nodes) == 0
+    p, got, f, st = ctx.memberships(0)
+    assert np.array_equal(p, optr) and np.array_equal(got, onodes)
+    np.testing.assert_allclose(f, of, rtol=F_RTOL, atol=0)
+    assert np.array_equal(st[:, :6], ost[:, :6])
+    ctx.free_graph(gid)
