@@ -292,11 +292,20 @@ int dedup_scales(i64 *uoff, const i32 *ulen, const u64 *uhash, const double *uf,
         }
         return MSCD_OK;
     }
-    const int32_t step = (int32_t)std::min<i64>(S, std::max<i64>(1, BATCH_UNITS / N));
-    int rc = MSCD_OK;
-    for (int32_t s = 0; s < S && rc == MSCD_OK; s += step) {
+    int32_t step = (int32_t)std::min<i64>(S, std::max<i64>(1, BATCH_UNITS / N));
+    for (int32_t s = 0; s < S;) {
         const i64 u = (i64)s * N;
-        rc = dedup_batch(uoff + u, ulen + u, uhash + u, uf + u, nodes, N, std::min(step, S - s), out + s, st);
+        const int32_t m = std::min(step, S - s);
+        const int rc = dedup_batch(uoff + u, ulen + u, uhash + u, uf + u, nodes, N, m, out + s, st);
+        if (rc == MSCD_ENOMEM && m > 1) {
+            // less memory free than a batch takes: scale by scale (a batch
+            // changes nothing before it has all its memory)
+            cudaGetLastError();
+            step = 1;
+            continue;
+        }
+        if (rc) return rc;
+        s += m;
     }
-    return rc;
+    return MSCD_OK;
 }

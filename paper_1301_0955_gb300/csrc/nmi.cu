@@ -922,16 +922,24 @@ int nmi_chain(const ScaleResult *sc, int32_t S, i64 n, const i64 *part_off, int3
         if ((rc = dev_alloc(&acc, (i64)h.size(), st))) break;
         if ((rc = cuda_status(cudaMemsetAsync(acc, 0, h.size() * sizeof(acc[0]), st)))) break;
         // as many scales at a time as CHUNK_SCRATCH bytes hold (two at least);
-        // a scale without communities ends a run of pairs
+        // a scale without communities ends a run of pairs.  Where the device has
+        // less memory free than that, two scales at a time.
+        int32_t at_most = CHUNK_SCALES;
         for (int32_t s0 = 0; s0 + 1 < S && rc == MSCD_OK;) {
             int32_t s1 = s0;
             size_t bytes = 0;
             while (s1 < S && sc[s1].n_comms > 0) {
                 bytes += scale_scratch(sc[s1], n, P);
-                if (s1 - s0 >= 2 && (bytes > CHUNK_SCRATCH || s1 - s0 >= CHUNK_SCALES)) break;
+                if (s1 - s0 >= 2 && (bytes > CHUNK_SCRATCH || s1 - s0 >= at_most)) break;
                 ++s1;
             }
             if (s1 - s0 >= 2) rc = chunk_terms(sc + s0, s1 - s0, n, part_off, P, tab, acc + words * s0, st);
+            if (rc == MSCD_ENOMEM && s1 - s0 > 2) {
+                cudaGetLastError();
+                at_most = 2;
+                rc = MSCD_OK;
+                continue;
+            }
             // the last scale of a chunk is the first of the next one
             s0 = s1 < S && sc[s1].n_comms <= 0 ? s1 + 1 : std::max(s1 - 1, s0 + 1);
             if (s1 == S) break;
