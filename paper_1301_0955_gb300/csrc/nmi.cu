@@ -55,6 +55,7 @@
 // are only ever taken from the same part, and the means run over each part's
 // communities.
 #include <algorithm>
+#include <list>
 #include <vector>
 
 #include "common.cuh"
@@ -755,9 +756,14 @@ struct Rooms {
 // The pairs of the successive scales sc[0..ns) (each with communities) into
 // acc (6 P words per pair, zero): every step is one launch over all of them.
 // Waits for the stream only where a community may meet more partners than a
-// CTA's table holds.
+// CTA's table holds; what it copies from the host goes into `tables`, to be kept
+// until the stream has been waited for.
+struct Tables {
+    std::vector<Scale> scales;
+    std::vector<Direction> dirs;
+};
 int chunk_terms(const ScaleResult *sc, int ns, i64 n, const i64 *part_off, int32_t P, const double *tab,
-                unsigned long long *acc, cudaStream_t st) {
+                unsigned long long *acc, Tables &tables, cudaStream_t st) {
     const int np = ns - 1, nd = 2 * np;
     i64 most = 0, most_m = 0;
     for (int s = 0; s < ns; ++s) {
@@ -785,8 +791,10 @@ int chunk_terms(const ScaleResult *sc, int ns, i64 n, const i64 *part_off, int32
     i64 entries = 0;
     for (int s = 0; s < ns; ++s) entries += sc[s].n_nodes;
     const size_t o_mlist = R.take((size_t)entries * 4);
-    std::vector<Scale> scales(ns);
-    std::vector<Direction> dirs(nd);
+    std::vector<Scale> &scales = tables.scales;
+    std::vector<Direction> &dirs = tables.dirs;
+    scales.assign(ns, Scale{});
+    dirs.assign(nd, Direction{});
     std::vector<size_t> o_s(3 * ns), o_d(6 * nd);
     for (int s = 0; s < ns; ++s) {
         const size_t C = (size_t)sc[s].n_comms;
@@ -913,6 +921,7 @@ int nmi_chain(const ScaleResult *sc, int32_t S, i64 n, const i64 *part_off, int3
     unsigned long long *acc = nullptr;
     const size_t words = 6 * (size_t)P;
     std::vector<unsigned long long> h(words * pairs);
+    std::list<Tables> tables;
     int rc = MSCD_OK;
     do {
         if (n <= TERMS_MAX) {
@@ -933,7 +942,10 @@ int nmi_chain(const ScaleResult *sc, int32_t S, i64 n, const i64 *part_off, int3
                 if (s1 - s0 >= 2 && (bytes > CHUNK_SCRATCH || s1 - s0 >= at_most)) break;
                 ++s1;
             }
-            if (s1 - s0 >= 2) rc = chunk_terms(sc + s0, s1 - s0, n, part_off, P, tab, acc + words * s0, st);
+            if (s1 - s0 >= 2) {
+                tables.emplace_back();
+                rc = chunk_terms(sc + s0, s1 - s0, n, part_off, P, tab, acc + words * s0, tables.back(), st);
+            }
             if (rc == MSCD_ENOMEM && s1 - s0 > 2) {
                 cudaGetLastError();
                 at_most = 2;
