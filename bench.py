@@ -47,8 +47,8 @@ N_SCALES = 20  # the full method's workload (lfr-100k)
 WORKLOAD = ("lfr-100k: 100,000-node LFR-style hierarchical graph (degrees power-law 2.5, mean 20, max 200; "
             "community sizes 20-1000 power-law 1.5; 2 levels, mixing 0.3/0.1; unweighted, seed 1), "
             "20 log-spaced scales in [0.5,1], every node a seed")
-GROW_SOURCES = ["paper_1301_0955_gb300/csrc/grow.cu", "paper_1301_0955_gb300/csrc/exact.cuh",
-                "paper_1301_0955_gb300/csrc/grow.cuh"]
+GROW_SOURCES = ["paper_1301_0955_gb300/csrc/grow_kernel.cuh", "paper_1301_0955_gb300/csrc/exact.cuh",
+                "paper_1301_0955_gb300/csrc/grow.cuh", "paper_1301_0955_gb300/csrc/ladder.cu"]
 # DRAM traffic of the growth kernel per workload (ncu capture, see profiles/)
 PROFILE_FILES = {"lfr-100k": os.path.join(ROOT, "profiles", "grow_kernel_lfr100k_traffic.json"),
                  "lfr-1m-weighted": os.path.join(ROOT, "profiles", "grow_kernel_lfr1m_weighted_traffic.json")}

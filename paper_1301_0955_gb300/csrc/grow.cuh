@@ -7,9 +7,10 @@
 #define GROW_SMEM_MAX (220 * 1024)  // dynamic shared memory of a CTA of a shared-memory class, at most
 // Global-arena classes: threads per CTA, and the CTAs an SM has registers for.
 // Up to 32,768 slots the loop's 80 registers let 24 units share an SM: on the
-// 1-of-80 weighted 1M-node run the 8,192-slot class takes 283 ms, 316 at 16
-// units (128 registers), 278 at 32 (64, spilling a little; slower than 24
-// where few units run).  The few units of the wider classes take 128.
+// 1-of-80 weighted 1M-node run the 8,192-slot class took 283 ms with them, 316
+// at 16 units (128 registers), 278 at 32 (64, spilling a little; slower than 24
+// where few units run); with the present slots and tests 275, and 286 at 20
+// units (96, without spills).  The few units of the wider classes take 128.
 #define GROW_CTA_SMEM (size_t)6144  // a CTA's static shared memory and what the system takes, at most
 #define GROW_SM_SMEM (size_t)(228 * 1024)
 #define GLOBAL_CTA_THREADS 128

@@ -69,8 +69,8 @@
 // in shared memory: with all of it inlined the kernel wanted 160 registers,
 // spilled in the loop at 16 units per SM and waited for instructions.  Growth
 // of the 1-of-8 run of the 100,000-node graph (250,000 units, the shared class
-// and the 8,192-slot one): 48 + 237 ms before, 28 + 151 now; of the 1-of-80 run
-// of the weighted 1M-node graph 41 + 461, now 29 + 280.
+// and the 8,192-slot one): 48 + 237 ms before, 26 + 139 now; of the 1-of-80 run
+// of the weighted 1M-node graph 41 + 461, now 28 + 272.
 #pragma once
 
 #include <algorithm>
@@ -185,7 +185,7 @@ struct Slots {  // unweighted
 // groups can afford; a visit is one sector and a 2-byte store, and 15 states
 // instead of 12 fit an SM's shared memory.  Against keys in the slots (12 bytes):
 // the shared class of the 10,000-node run 27.7 -> 23.9 ms, of the 1,000-node run
-// 1.69 -> 1.37, the 8,192-slot class of the union of 12 graphs 208 -> 193, of the
+// 1.69 -> 1.37 ms, the 8,192-slot class of the union of 12 graphs 208 -> 193, of the
 // 1-of-8 run of the 100,000-node graph 156 -> 151.
 template <>
 struct Slots<u16, false> {

@@ -1,4 +1,4 @@
-// The growth kernels of unweighted graphs with every degree below 2^16.
+// The growth kernels of unweighted graphs with every degree below 2^15.
 #include "grow_kernel.cuh"
 
 int grow_launch_u16(const GrowArgs &a, int blocks, int threads, size_t smem, cudaStream_t st, int *occ) {
