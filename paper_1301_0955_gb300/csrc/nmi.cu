@@ -531,6 +531,9 @@ __global__ void __launch_bounds__(BLK_WARPS * 32) pairs_block(const __grid_const
         for (i64 e = e0 + w * step; e < e1; e += BLK_WARPS * step) {
             if (*(volatile int *)&over) break;
             visit_lists(d.A.nodes, e, min(e + step, e1), d.B.mptr, d.B.mlist, [&](i32 l) {
+                // (a table past half full is given up at once: filled up, each
+                // look-up would pass all of it)
+                if (*(volatile int *)&over) return;
                 u32 h;
                 if (C.add(l, h)) {
                     const int f = atomicAdd(&fill, 1);
