@@ -24,8 +24,12 @@ enum : u32 {
     CAT_RANGE = 64u,
 };
 
+// What each kernel finds goes into a word of its own, which only later kernels
+// read: blocks of one kernel must not act on what its other blocks have found so far.
 struct PrepState {
-    u32 mask;
+    u32 rows;                      // of check_row_ptr: CAT_STRUCT
+    u32 mask;                      // of check_entries
+    u32 range;                     // of the degree kernels: CAT_RANGE
     int min_lowbit;
     unsigned long long total;      // exact volume (valid while total_d < 2^63)
     double total_d;                // coarse volume (within 1%), guards against wrap-around
@@ -38,7 +42,7 @@ __global__ void check_row_ptr(const i64 *rp, i64 n, i64 nnz, PrepState *ps) {
     if (u > n) return;
     bool bad = (u == 0) ? (rp[0] != 0) : (rp[u] < rp[u - 1]);
     if (u == n) bad = bad || rp[n] != nnz;
-    if (bad) atomicOr(&ps->mask, CAT_STRUCT);
+    if (bad) atomicOr(&ps->rows, CAT_STRUCT);
 }
 
 // lowbit exponent of a positive finite FP32 value: w = odd * 2^lowbit
@@ -60,7 +64,7 @@ __device__ __forceinline__ int f32_lowbit(float w, u32 *odd) {
 // none is left over.  The look-ups (a binary search each) are what the kernel
 // takes its time for: half of them, 969 -> 600 us for 27 million entries.
 __global__ void check_entries(const i64 *rp, const i32 *col, const float *w, i64 n, PrepState *ps) {
-    if (*(volatile u32 *)&ps->mask) return;  // the row pointers cannot be followed
+    if (ps->rows) return;  // the row pointers cannot be followed
     const int lane = threadIdx.x & 31;
     const i64 warps = (i64)gridDim.x * (blockDim.x >> 5);
     u32 mask = 0;
@@ -163,7 +167,7 @@ __device__ __forceinline__ void add_totals(unsigned long long tot, float tot_f, 
 
 // Unweighted: thread per row, k_u = its entries.
 __global__ void degrees(const i64 *rp, i64 n, i64 *k, float *logk, PrepState *ps) {
-    if (*(volatile u32 *)&ps->mask) return;
+    if (ps->rows | ps->mask) return;
     unsigned long long tot = 0, kmax = 0;
     for (i64 u = (i64)blockIdx.x * blockDim.x + threadIdx.x; u < n; u += (i64)gridDim.x * blockDim.x) {
         const i64 s = rp[u + 1] - rp[u];
@@ -181,10 +185,10 @@ __global__ void degrees(const i64 *rp, i64 n, i64 *k, float *logk, PrepState *ps
 // entry moves: 170 us for 27 million, 69 + 622 us as a pass for the
 // weights and one for the sums with a binary64 guard.
 __global__ void weighted_degrees(const i64 *rp, const float *w, i64 n, i64 *wfx, i64 *k, float *logk, PrepState *ps) {
-    if (*(volatile u32 *)&ps->mask) return;
+    if (ps->rows | ps->mask) return;
     constexpr int ROW = 16;
     const int lane = threadIdx.x & (ROW - 1);
-    const int ue = *(volatile int *)&ps->min_lowbit;
+    const int ue = ps->min_lowbit;
     const i64 rows = (i64)gridDim.x * (blockDim.x / ROW);
     const i64 steps = (n + rows - 1) / rows;
     unsigned long long tot = 0, kmax = 0;
@@ -220,7 +224,7 @@ __global__ void weighted_degrees(const i64 *rp, const float *w, i64 n, i64 *wfx,
             kmax = max(kmax, s);
         }
     }
-    if (mask) atomicOr(&ps->mask, mask);
+    if (mask) atomicOr(&ps->range, mask);
     add_totals(tot, tot_f, kmax, ps);
 }
 
@@ -240,7 +244,7 @@ int first_category(u32 mask) {
 int graph_prepare(i64 n, i64 nnz, const i64 *rp, const i32 *col, const float *w, i64 *wfx, i64 *k, float *logk,
                   DevGraph *g, cudaStream_t st) {
     PrepState *ps = nullptr;
-    const PrepState init{0u, INT32_MAX, 0ull, 0.0, 0ull, 0ull};
+    const PrepState init{0u, 0u, 0u, INT32_MAX, 0ull, 0.0, 0ull, 0ull};
     MSCD_CUDA(cudaMallocAsync((void **)&ps, sizeof(PrepState), st));
     int rc = MSCD_OK;
     PrepState h{};
@@ -262,9 +266,9 @@ int graph_prepare(i64 n, i64 nnz, const i64 *rp, const i32 *col, const float *w,
         if ((rc = cuda_status(cudaMemcpyAsync(&h, ps, sizeof(h), cudaMemcpyDeviceToHost, st)))) break;
         if ((rc = cuda_status(cudaStreamSynchronize(st)))) break;
         if ((rc = cuda_status(cudaGetLastError()))) break;
-        // CAT_RANGE comes after the symmetry found by the count
-        if (!(h.mask & ~(u32)CAT_RANGE) && h.below) h.mask |= CAT_NOTSYM;
-        if ((rc = first_category(h.mask))) break;
+        u32 found = h.rows | h.mask;
+        if (!found && h.below) found = CAT_NOTSYM;
+        if ((rc = first_category(found | h.range))) break;
         if (h.total_d >= 0x1p63 || h.total >= (1ull << 62)) { rc = MSCD_ERANGE; break; }
         g->n = n;
         g->nnz = nnz;
