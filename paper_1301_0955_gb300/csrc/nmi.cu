@@ -529,7 +529,9 @@ __global__ void __launch_bounds__(BLK_WARPS * 32) pairs_block(const __grid_const
         const i32 k = d.active[q];
         const i64 e0 = d.A.ptr[k], e1 = d.A.ptr[k + 1], step = member_chunk(e1 - e0, BLK_WARPS);
         for (i64 e = e0 + w * step; e < e1; e += BLK_WARPS * step) {
-            if (*(volatile int *)&over) break;
+            // decided for the warp as a whole: visit_lists is warp-collective, and
+            // other warps raise the flag at any time
+            if (__any_sync(FULL_MASK, *(volatile int *)&over)) break;
             visit_lists(d.A.nodes, e, min(e + step, e1), d.B.mptr, d.B.mlist, [&](i32 l) {
                 // (a table past half full is given up at once: filled up, each
                 // look-up would pass all of it)

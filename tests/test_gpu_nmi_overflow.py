@@ -1,0 +1,27 @@
+"""GPU: communities whose partners overflow a CTA's count table (4,096) while all
+of its warps are still walking members, in turn with communities that fit the
+table the first ones leave behind.  Against the oracle."""
+import numpy as np
+import pytest
+
+from test_gpu_nmi import ctx  # noqa: F401
+from test_gpu_nmi_tiers import cover, pick
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("partners,size", [(9000, 5), (20000, 4), (5200, 3)])
+def test_table_overflow_amid_the_walk(orc, ctx, partners, size):
+    r = np.random.default_rng(partners)
+    n = 12000
+    # 2,000 members overflow the table (in the third case some of 2,000, all of
+    # 12,000 do), 700 fit it, 4 fit a warp's
+    a = [np.arange(2000 * i, 2000 * (i + 1)) for i in range(6)]
+    a += [pick(r, n, 700) for _ in range(40)] + [pick(r, n, 2000) for _ in range(12)] + [pick(r, n, 4)]
+    a += [np.arange(n)]
+    b = [pick(r, n, size) for _ in range(partners)]
+    a, b = cover(a), cover(b)
+    want = orc.nmi(n, a[0], a[1], b[0], b[1])
+    for _ in range(3):
+        assert ctx.nmi_covers(n, a, b) == pytest.approx(want, abs=1e-12)
+    assert ctx.nmi_covers(n, b, a) == pytest.approx(want, abs=1e-12)
