@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(REACH_WARPS * 32) reach_smem(const i64 *cptr, 
                     if (f >= REACH_TABLE / 2) over = true;
                     else used[f] = (unsigned short)h;
                 }
-            });
+            }, [] { return false; });
             over = __any_sync(FULL_MASK, over);
         }
         __syncwarp();
@@ -291,7 +291,7 @@ __global__ void reach_global(const i64 *cptr, const i32 *cnodes, const i64 *mptr
             visit_lists(cnodes, e, min(e + 32, e1), mptr, mlist, [&](i32 o) {
                 u32 h;
                 if (o != c) count_in(keys, cnts, tm, o, h);
-            });
+            }, [] { return false; });
         __syncwarp();
         unsigned long long best = ~0ull;
         for (u32 t0 = 0; t0 <= tm; t0 += 32) {

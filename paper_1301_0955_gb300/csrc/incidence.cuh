@@ -7,9 +7,12 @@
 // in nodes[e0, e1), at most 32 nodes.  The lists are laid end to end: the lanes
 // take 32 entries of several lists at a time, and the next ones are loaded
 // while these are handled (lists are often shorter than a warp is wide, and one
-// at a time each costs three dependent loads).  Warp-collective.
-template <class F>
-__device__ __forceinline__ void visit_lists(const i32 *nodes, i64 e0, i64 e1, const i64 *mptr, const i32 *mlist, F f) {
+// at a time each costs three dependent loads).  After every 32 * AHEAD entries
+// the lanes ask done(); if it is true for any of them the warp leaves, and true
+// is returned to all.  Warp-collective.
+template <class F, class D>
+__device__ __forceinline__ bool visit_lists(const i32 *nodes, i64 e0, i64 e1, const i64 *mptr, const i32 *mlist, F f,
+                                            D done) {
     constexpr int AHEAD = 4;  // entries a lane has in flight
     const int lane = threadIdx.x & 31;
     i64 lo = 0, n = 0;
@@ -21,9 +24,12 @@ __device__ __forceinline__ void visit_lists(const i32 *nodes, i64 e0, i64 e1, co
     if (__any_sync(FULL_MASK, n > 1 << 25)) {  // the sums below would not fit
         for (int i = 0; i < 32; ++i) {
             const i64 b = __shfl_sync(FULL_MASK, lo, i), m = __shfl_sync(FULL_MASK, n, i);
-            for (i64 t = lane; t < m; t += 32) f(mlist[b + t]);
+            for (i64 t = 0; t < m; t += 32) {
+                if (t + lane < m) f(mlist[b + t + lane]);
+                if (__any_sync(FULL_MASK, done())) return true;
+            }
         }
-        return;
+        return false;
     }
     const int len = (int)n;
     int incl = len;  // node i's entries are incl - len .. incl of the whole
@@ -50,5 +56,7 @@ __device__ __forceinline__ void visit_lists(const i32 *nodes, i64 e0, i64 e1, co
 #pragma unroll
         for (int j = 0; j < AHEAD; ++j)
             if (l[j] >= 0) f(l[j]);
+        if (__any_sync(FULL_MASK, done())) return true;
     }
+    return false;
 }

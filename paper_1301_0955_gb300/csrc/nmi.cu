@@ -441,17 +441,17 @@ __global__ void __launch_bounds__(NMI_WARPS * 32) pairs_warp(const __grid_consta
         if (!over) {
             if (lane == 0) sfill[w] = 0;
             __syncwarp();
-            for (i64 e = e0; e < e1 && !over; e += 32) {
-                visit_lists(d.A.nodes, e, min(e + 32, e1), d.B.mptr, d.B.mlist, [&](i32 l) {
+            // (a table past half full is given up within 128 entries: filled up, each
+            // look-up would pass all of it)
+            for (i64 e = e0; e < e1 && !over; e += 32)
+                over = visit_lists(d.A.nodes, e, min(e + 32, e1), d.B.mptr, d.B.mlist, [&](i32 l) {
                     u32 h;
                     if (C.add(l, h)) {
                         const int f = atomicAdd(&sfill[w], 1);
                         if (f >= NMI_TABLE / 2) over = true;
                         else used[f] = (unsigned short)h;
                     }
-                });
-                over = __any_sync(FULL_MASK, over);
-            }
+                }, [&] { return over; });
             __syncwarp();
             if (over) {  // more buckets than listed: clear all
                 for (int t = lane; t < NMI_TABLE; t += 32) {
@@ -529,20 +529,16 @@ __global__ void __launch_bounds__(BLK_WARPS * 32) pairs_block(const __grid_const
         const i32 k = d.active[q];
         const i64 e0 = d.A.ptr[k], e1 = d.A.ptr[k + 1], step = member_chunk(e1 - e0, BLK_WARPS);
         for (i64 e = e0 + w * step; e < e1; e += BLK_WARPS * step) {
-            // decided for the warp as a whole: visit_lists is warp-collective, and
-            // other warps raise the flag at any time
-            if (__any_sync(FULL_MASK, *(volatile int *)&over)) break;
-            visit_lists(d.A.nodes, e, min(e + step, e1), d.B.mptr, d.B.mlist, [&](i32 l) {
-                // (a table past half full is given up at once: filled up, each
-                // look-up would pass all of it)
-                if (*(volatile int *)&over) return;
-                u32 h;
-                if (C.add(l, h)) {
-                    const int f = atomicAdd(&fill, 1);
-                    if (f >= BLK_TABLE / 2) over = 1;
-                    else used[f] = (unsigned short)h;
-                }
-            });
+            // (also here, each warp within 128 entries)
+            if (visit_lists(d.A.nodes, e, min(e + step, e1), d.B.mptr, d.B.mlist, [&](i32 l) {
+                    u32 h;
+                    if (C.add(l, h)) {
+                        const int f = atomicAdd(&fill, 1);
+                        if (f >= BLK_TABLE / 2) over = 1;
+                        else used[f] = (unsigned short)h;
+                    }
+                }, [&] { return *(volatile int *)&over != 0; }))
+                break;
         }
         __syncthreads();
         if (over) {
@@ -595,7 +591,7 @@ __global__ void __launch_bounds__(GLB_WARPS * 32) pairs_global(const __grid_cons
             visit_lists(d.A.nodes, e, min(e + step, e1), d.B.mptr, d.B.mlist, [&](i32 l) {
                 u32 h;
                 if (C.add(l, h)) used[atomicAdd(fill, 1u)] = (i32)h;
-            });
+            }, [] { return false; });
         __syncthreads();
         // only the claimed buckets, emptied again for the table's next user
         const u32 nf = *(volatile unsigned int *)fill;

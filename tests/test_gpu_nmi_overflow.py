@@ -25,3 +25,20 @@ def test_table_overflow_amid_the_walk(orc, ctx, partners, size):
     for _ in range(3):
         assert ctx.nmi_covers(n, a, b) == pytest.approx(want, abs=1e-12)
     assert ctx.nmi_covers(n, b, a) == pytest.approx(want, abs=1e-12)
+
+
+@pytest.mark.parametrize("met", [255, 256, 257, 384, 512, 700])
+def test_few_members_many_partners(orc, ctx, met):
+    """Communities of 11 members that all lie in the same `met` partners: a warp's
+    table (512 entries, listed up to 256) is at its limit before the first
+    members have been walked, and what comes after must still be counted where it
+    is not given up."""
+    r = np.random.default_rng(met)
+    n = 3000
+    core = np.arange(40)
+    a = [pick(r, 40, 11) for _ in range(60)] + [pick(r, n, 30) for _ in range(20)]
+    b = [np.concatenate([core, 40 + pick(r, n - 40, 1 + i % 90)]) for i in range(met)]
+    a, b = cover(a), cover(b)
+    want = orc.nmi(n, a[0], a[1], b[0], b[1])
+    assert ctx.nmi_covers(n, a, b) == pytest.approx(want, abs=1e-12)
+    assert ctx.nmi_covers(n, b, a) == pytest.approx(want, abs=1e-12)
