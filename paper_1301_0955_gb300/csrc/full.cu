@@ -238,17 +238,17 @@ __global__ void __launch_bounds__(REACH_WARPS * 32) reach_smem(const i64 *cptr, 
         __syncwarp();
         bool over = false;
         const i64 e1 = cptr[c + 1];
-        for (i64 e = cptr[c]; e < e1 && !over; e += 32) {
-            visit_lists(cnodes, e, min(e + 32, e1), mptr, mlist, [&](i32 o) {
+        // (a table past half full is given up within 128 entries: filled up, each
+        // look-up would pass all of it)
+        for (i64 e = cptr[c]; e < e1 && !over; e += 32)
+            over = visit_lists(cnodes, e, min(e + 32, e1), mptr, mlist, [&](i32 o) {
                 u32 h;
                 if (o != c && count_in(keys, cnts, REACH_TABLE - 1, o, h)) {
                     const int f = atomicAdd(&sfill[w], 1);
                     if (f >= REACH_TABLE / 2) over = true;
                     else used[f] = (unsigned short)h;
                 }
-            }, [] { return false; });
-            over = __any_sync(FULL_MASK, over);
-        }
+            }, [&] { return over; });
         __syncwarp();
         if (over) {
             if (lane == 0) spill[atomicAdd(n_spill, 1ull)] = c;
