@@ -239,8 +239,11 @@ int grow_units(GrowPipe &w, const GrowArgs &proto, i64 n_units, const std::vecto
             // one statically mapped unit per warp: a grid over the items
             const int wpc = threads / 32;
             for (i64 b = 0; b < n_work && rc == MSCD_OK; b += chunk) {
-                a.work_base = b;
+                // (the last CTA's warps beyond the chunk find no item: theirs belong
+                // to the next launch)
                 const i64 items = std::min<i64>(chunk, n_work - b);
+                a.work_base = b;
+                a.n_work = b + items;
                 rc = grow_launch(a, (int)((items + wpc - 1) / wpc), threads, smem, st);
             }
         }
