@@ -7,6 +7,11 @@
 namespace {
 
 constexpr i64 MIDDLE_SLOTS = 16384;
+// Classes eight times the last one, but none of these is left out (see make_ladder).
+constexpr i64 WIDE_SLOTS = 131072;
+constexpr i64 WIDE_ROUNDS = 3;
+constexpr i64 KEPT_SLOTS[] = {MIDDLE_SLOTS, 65536, WIDE_SLOTS, 524288};
+constexpr size_t ARENA_BUDGET = (size_t)4 << 30;  // states of a launch, at most
 
 struct Task {
     int cls;                 // index in the ladder
@@ -96,12 +101,21 @@ int make_ladder(const DevGraph &G, i64 max_part_n, const mscd_params &p, std::ve
     i64 cg = ladder->back();
     bool first = true;
     while (cg < full) {
-        // Eight times the last class, but 16,384 slots before the wide classes:
-        // up to there the buckets are 4 bytes and the group bounds leave most of
-        // the SM's shared memory to the L1 cache.  The 2,293 units of the 1-of-80
-        // run of the weighted 1M-node graph that touch more than 8,192 nodes take
-        // 34 ms at 16,384 slots, 41 at 32,768 and 52 at 65,536.
-        i64 next = cg >= MIDDLE_SLOTS / 4 && cg < MIDDLE_SLOTS ? MIDDLE_SLOTS : cg * 8;
+        // 16,384 slots come before the wide classes: up to there the buckets are 4
+        // bytes and the group bounds leave most of the SM's shared memory to the L1
+        // cache.  The 2,293 units of the 1-of-80 run of the weighted 1M-node graph
+        // that touch more than 8,192 nodes take 34 ms at 16,384 slots, 41 at 32,768
+        // and 52 at 65,536.  Among the wide ones a state of 65,536 weighted slots is
+        // 2.4 MB, of 131,072 4.8: long lists need the smaller one, as the arena holds
+        // 1,807 or 903 units (22,112 units that touch up to 140,000 nodes of a weighted
+        // 300,000-node graph: 9.1 s with it, 13.3 without), and short ones skip it
+        // (see grow_units).
+        i64 next = cg * 8;
+        for (const i64 v : KEPT_SLOTS)
+            if (v > cg && v < next) {
+                next = v;
+                break;
+            }
         if (first && p.global_slots > cg) next = p.global_slots;
         first = false;
         cg = std::min<i64>(next, full);
@@ -132,6 +146,20 @@ int grow_units(GrowPipe &w, const GrowArgs &proto, i64 n_units, const std::vecto
         // memory, where the smaller class fits.
         if (!plain && t.cls > 0 && n_work > w.sm_count && n_work <= (i64)w.sm_count * w.p.global_warps_per_sm)
             while (!in_smem[t.cls] && t.cls + 1 < (int)ladder.size() && ladder[t.cls + 1] <= MIDDLE_SLOTS) ++t.cls;
+        // Among the wide classes up to WIDE_ROUNDS times as many units as are resident
+        // at WIDE_SLOTS go there at once: 547 weighted units of which three outgrow
+        // 65,536 slots take 1.2 s, 1.1 + 1.1 one class after the other.  Longer lists
+        // gain more from the smaller states: 131,072 slots at once against 65,536
+        // first, ms, 1,446 / 2,390 / 3,923 unweighted units (1,159 resident) 382 and
+        // 413 / 557 and 449 / 791 and 606; 1,830 / 3,672 / 5,483 weighted ones (903
+        // resident) 1,879 and 2,695 / 3,142 and 3,444 / 4,195 and 3,798.
+        if (!plain && t.cls > 0)
+            while (!in_smem[t.cls] && ladder[t.cls] > MIDDLE_SLOTS && t.cls + 1 < (int)ladder.size() &&
+                   ladder[t.cls + 1] <= WIDE_SLOTS &&
+                   n_work <= WIDE_ROUNDS *
+                                 std::min<i64>((i64)(ARENA_BUDGET / grow_state_bytes(G, ladder[t.cls + 1], false)),
+                                               (i64)w.sm_count * WIDE_MIN_BLOCKS * GLOBAL_CTA_THREADS / 32))
+                ++t.cls;
         const int cap = ladder[t.cls];
         // A few left-over units (at most one an SM) run in shared memory where a
         // state of their class fits it: there is nothing to hide an arena's
@@ -218,9 +246,8 @@ int grow_units(GrowPipe &w, const GrowArgs &proto, i64 n_units, const std::vecto
                     smem = (size_t)wpc * bounds;
                 }
             }
-            const size_t budget = (size_t)4 << 30;
-            i64 warps = std::max<i64>(1, std::min<i64>((i64)(budget / a.state_bytes), (i64)w.sm_count * per_sm_warps));
-            if (plain) warps = (i64)(budget / a.state_bytes);
+            i64 warps = std::max<i64>(1, std::min<i64>((i64)(ARENA_BUDGET / a.state_bytes), (i64)w.sm_count * per_sm_warps));
+            if (plain) warps = (i64)(ARENA_BUDGET / a.state_bytes);
             warps = std::max<i64>(1, std::min<i64>(warps, std::max<i64>(n_work, 1)));
             if (plain) chunk = warps;
             threads = (int)std::min<i64>(warps, wpc) * 32;

@@ -40,9 +40,9 @@ void pipe_free(GrowPipe &w);
 void pipe_release_output(GrowPipe &w);
 
 // The ladder of node-slot capacities for a graph whose parts hold at most
-// max_part_n nodes: shared-memory classes, then global arenas of 8,192 slots,
-// 16,384 and growing 8x up to the first power of two above max_part_n (a class
-// that never overflows).
+// max_part_n nodes: shared-memory classes, then global arenas of 8,192, 16,384,
+// 65,536, 131,072 and 524,288 slots and growing 8x up to the first power of two
+// above max_part_n (a class that never overflows).
 int make_ladder(const DevGraph &G, i64 max_part_n, const mscd_params &p, std::vector<int> *ladder,
                 std::vector<bool> *in_smem);
 
