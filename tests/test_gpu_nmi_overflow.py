@@ -42,3 +42,18 @@ def test_few_members_many_partners(orc, ctx, met):
     want = orc.nmi(n, a[0], a[1], b[0], b[1])
     assert ctx.nmi_covers(n, a, b) == pytest.approx(want, abs=1e-12)
     assert ctx.nmi_covers(n, b, a) == pytest.approx(want, abs=1e-12)
+
+
+@pytest.mark.parametrize("lists", [63, 64, 65, 127, 128, 129])
+def test_lists_about_the_line_between_the_walks(orc, ctx, lists):
+    """Every node in exactly `lists` communities of the second cover (64 entries a
+    list is the line, 128 a step); communities of 1 to 70 members, so that the last
+    32 of them are fewer."""
+    r = np.random.default_rng(lists)
+    n = 480
+    a = [pick(r, n, m) for m in (1, 2, 31, 32, 33, 63, 64, 65, 70)] + [pick(r, n, 200)]
+    b = [p for _ in range(lists) for p in np.split(r.permutation(n), [40, 160, 170])]
+    a, b = cover(a), cover([np.sort(x) for x in b])
+    want = orc.nmi(n, a[0], a[1], b[0], b[1])
+    assert ctx.nmi_covers(n, a, b) == pytest.approx(want, abs=1e-12)
+    assert ctx.nmi_covers(n, b, a) == pytest.approx(want, abs=1e-12)
