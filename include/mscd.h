@@ -360,13 +360,18 @@ const char *mscd_last_error(mscd_ctx *ctx);
  * Limits and errors: MSCD_ERANGE for more than 2^20 units or 256 scales in
  * one call, and for a unit that touches more than 8192 nodes (the per-unit
  * slot arena of the array); MSCD_ESMALL when out_cap < *n_nodes_needed;
- * MSCD_EINVAL for bad arguments or seeds.  The array holds the states of
- * about 270 (weighted graphs) to 380 (unweighted) units at once, so a call
- * keeps a fraction of a large GPU busy: it suits small and medium batches.
+ * MSCD_EINVAL for bad arguments or seeds.  Units grow in shared memory first,
+ * on the whole GPU: 1,024 slots, then 4,096 for those that outgrow them.  What
+ * outgrows these runs in the array, which holds 336 states at once (232 for
+ * weighted graphs and for degrees from 32,768), so a call of many such units
+ * keeps a fraction of a large GPU busy.
  * The call waits for its stream (cudaStreamSynchronize) after the seed check,
- * when seeds are given, and once more to read its counters back; it returns
- * with the outputs written.  The first call on a device looks up the array's
- * device address once (make that first call before any stream capture).
+ * when seeds are given, and after each of the up to three launches to read its
+ * counters back; it returns with the outputs written.  The first call on a
+ * device also looks up the array's device address and launches every kernel
+ * that later calls may need once, with no work, and waits for them: later
+ * calls load no code and reserve no memory (make that first call before any
+ * stream capture).
  * Every call reuses the same array, which keeps the previous call's contents
  * (the call clears what must start at zero): calls that overlap on the GPU,
  * on any stream or context of one device, race on it and must not be

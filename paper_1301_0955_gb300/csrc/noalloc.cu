@@ -13,7 +13,10 @@
 //
 // Host code only ever sees a stand-in for that array's name; the device
 // address is taken once per device with cudaGetSymbolAddress (with the device
-// current) on the first call on that device, and passed to the kernel.
+// current) on the first call on that device, and passed to the kernel.  That
+// first call also runs every kernel that a later one may need (which depends on
+// its graph and on the units' sizes), without any work: the driver loads a
+// kernel's code, and reserves its local memory, when it is first launched.
 #include <cmath>
 #include <mutex>
 
@@ -56,6 +59,34 @@ __global__ void check_seeds_noalloc(const i32 *seeds, i64 N, i64 n, Header *hdr)
 // The scratch array (file scope, device memory of every GPU that loads the library).
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_BYTES];
 
+namespace {
+
+// Every kernel of mscd_grow_noalloc, launched with no work on st.
+int run_kernels_idle(unsigned char *base, cudaStream_t st) {
+    Header *hdr = (Header *)base;
+    MSCD_CUDA(cudaMemsetAsync(hdr, 0, offsetof(Header, alphas), st));
+    check_seeds_noalloc<<<1, 32, 0, st>>>(nullptr, 0, 0, hdr); note_launch();
+    // the slot types by the graph's largest degree and weights (see grow.cu)
+    const i64 kmax[] = {1, 32768, 1};
+    for (int type = 0; type < 3; ++type)
+        for (int smem = 0; smem < 2; ++smem) {
+            GrowArgs a{};
+            a.G.kmax = kmax[type];
+            a.G.wfx = type == 2 ? (const i64 *)base : nullptr;  // not read: there is no unit
+            a.work_counter = &hdr->work;
+            a.cap = 32;
+            a.use_smem = smem;
+            a.state_bytes = grow_state_bytes(a.G, a.cap, smem);
+            a.gstate = base + OFF_ARENA;
+            a.smem_per_warp = smem ? 0 : 8 * (size_t)(a.cap / 32);
+            const int rc = grow_launch(a, 1, 32, smem ? a.state_bytes : a.smem_per_warp, st);
+            if (rc) return rc;
+        }
+    return cuda_status(cudaStreamSynchronize(st));
+}
+
+}  // namespace
+
 extern "C" int mscd_grow_noalloc(mscd_ctx *ctx, int32_t graph_id, const double *alphas, int32_t n_scales,
                                  const int32_t *seeds, int64_t n_seeds, int32_t *out_nodes, int64_t out_cap,
                                  int64_t *out_offset, int32_t *out_len, double *out_fitness, int64_t *out_stats,
@@ -79,19 +110,22 @@ extern "C" int mscd_grow_noalloc(mscd_ctx *ctx, int32_t graph_id, const double *
     if (out_cap > 0 && !out_nodes) return MSCD_EINVAL;
     if (device < 0 || device >= MAX_DEVICES) return MSCD_EINVAL;
     MSCD_CUDA(cudaSetDevice(device));
-    // once per device, with that device current: the array's device address
+    cudaStream_t st = (cudaStream_t)cuda_stream;
+    // once per device, with that device current: the array's device address, and
+    // the kernels' code and local memory
     {
         std::lock_guard<std::mutex> lock(g_setup_mutex);
         if (!g_scratch_addr[device]) {
             void *p = nullptr;
             cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
             if (e != cudaSuccess) return cuda_status(e);
+            const int rc = run_kernels_idle((unsigned char *)p, st);
+            if (rc) return rc;
             g_scratch_addr[device] = p;
         }
     }
     unsigned char *base = (unsigned char *)g_scratch_addr[device];
     Header *hdr = (Header *)base;
-    cudaStream_t st = (cudaStream_t)cuda_stream;
     // the array keeps the previous call's contents: zero the header's counters
     MSCD_CUDA(cudaMemsetAsync(hdr, 0, offsetof(Header, alphas), st));
     MSCD_CUDA(cudaMemcpyAsync(hdr->alphas, alphas, n_scales * sizeof(double), cudaMemcpyHostToDevice, st));
