@@ -31,8 +31,7 @@ struct PrepState {
     u32 mask;                      // of check_entries
     u32 range;                     // of the degree kernels: CAT_RANGE
     int min_lowbit;
-    unsigned long long total;      // exact volume (valid while total_d < 2^63)
-    double total_d;                // coarse volume (within 1%), guards against wrap-around
+    unsigned long long total;      // exact volume (valid while `range` is 0)
     unsigned long long kmax;       // largest degree
     unsigned long long below;      // entries with a smaller column than their row, minus those with a larger one
 };
@@ -137,32 +136,35 @@ __global__ void check_entries(const i64 *rp, const i32 *col, const float *w, i64
     }
 }
 
-// The volume, the coarse volume and the largest degree of a block's rows: one
-// set of global atomics per block (they all meet on one address).
-__device__ __forceinline__ void add_totals(unsigned long long tot, float tot_f, unsigned long long kmax, PrepState *ps) {
+// s += v, both terms of sums that must stay below 2^62 (positive, so that one
+// that reaches it is out of range whatever else comes).  `high` collects the
+// upper words of the sums: from below 2^62 a sum reaches it in one addition of at
+// most 2^62, which sets bit 62 before any later one can wrap.
+__device__ __forceinline__ void add_seen(unsigned long long &s, unsigned long long v, u32 &high) {
+    s += v;
+    high |= (u32)(s >> 32);
+}
+
+// The volume and the largest degree of a block's rows: one set of global
+// atomics per block (they all meet on one address).
+__device__ __forceinline__ void add_totals(unsigned long long tot, unsigned long long kmax, u32 high, PrepState *ps) {
     __shared__ unsigned long long btot, bkmax;
-    __shared__ float btot_f;
-    if (threadIdx.x == 0) {
-        btot = bkmax = 0;
-        btot_f = 0.0f;
-    }
+    if (threadIdx.x == 0) btot = bkmax = 0;
     __syncthreads();
     for (int o = 16; o; o >>= 1) {
-        tot += __shfl_xor_sync(FULL_MASK, tot, o);
-        tot_f += __shfl_xor_sync(FULL_MASK, tot_f, o);
+        add_seen(tot, __shfl_xor_sync(FULL_MASK, tot, o), high);
         kmax = max(kmax, __shfl_xor_sync(FULL_MASK, kmax, o));
     }
     if ((threadIdx.x & 31) == 0) {
-        atomicAdd(&btot, tot);
-        atomicAdd(&btot_f, tot_f);
+        high |= (u32)((atomicAdd(&btot, tot) + tot) >> 32);
         atomicMax(&bkmax, kmax);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        atomicAdd(&ps->total, btot);
-        atomicAdd(&ps->total_d, (double)btot_f);
+        high |= (u32)((atomicAdd(&ps->total, btot) + btot) >> 32);
         atomicMax(&ps->kmax, bkmax);
     }
+    if (high >> 30) atomicOr(&ps->range, CAT_RANGE);
 }
 
 // Unweighted: thread per row, k_u = its entries.
@@ -176,14 +178,14 @@ __global__ void degrees(const i64 *rp, i64 n, i64 *k, float *logk, PrepState *ps
         tot += (unsigned long long)s;
         kmax = max(kmax, (unsigned long long)s);
     }
-    add_totals(tot, (float)tot, kmax, ps);
+    add_totals(tot, kmax, 0, ps);
 }
 
 // Weighted: half a warp per row writes the exact weights and sums them in the
-// same pass, k_u and log2 k_u.  A sum that might not fit 64 bits (binary32
-// guard, within 1%) is out of range whatever it is.  Bound by the 12 bytes an
-// entry moves: 170 us for 27 million, 69 + 622 us as a pass for the
-// weights and one for the sums with a binary64 guard.
+// same pass, k_u and log2 k_u.  Bound by the 12 bytes an entry moves: 170 us for
+// 27 million (69 + 622 us as a pass for the weights and one for the sums with a
+// binary64 guard against wrap-around; 205 with a comparison and a select at
+// every addition in place of add_seen's collected words).
 __global__ void weighted_degrees(const i64 *rp, const float *w, i64 n, i64 *wfx, i64 *k, float *logk, PrepState *ps) {
     if (ps->rows | ps->mask) return;
     constexpr int ROW = 16;
@@ -192,40 +194,31 @@ __global__ void weighted_degrees(const i64 *rp, const float *w, i64 n, i64 *wfx,
     const i64 rows = (i64)gridDim.x * (blockDim.x / ROW);
     const i64 steps = (n + rows - 1) / rows;
     unsigned long long tot = 0, kmax = 0;
-    float tot_f = 0.0f;
-    u32 mask = 0;
+    u32 high = 0;
     i64 u = (i64)blockIdx.x * (blockDim.x / ROW) + threadIdx.x / ROW;
     for (i64 step = 0; step < steps; ++step, u += rows) {
         unsigned long long s = 0;
-        float f = 0.0f;
         const i64 re = u < n ? rp[u + 1] : 0;
         for (i64 e = (u < n ? rp[u] : 0) + lane; e < re; e += ROW) {
-            const float x = w[e];
             u32 odd;
-            const int sh = f32_lowbit(x, &odd) - ue;  // >= 0
+            const int sh = f32_lowbit(w[e], &odd) - ue;  // >= 0
             const int len = 32 - __clz((int)odd);
             i64 v = 0;
             if ((odd == 1u) ? (sh <= 62) : (len + sh <= 62)) v = (i64)odd << sh;
-            else mask |= CAT_RANGE;
+            else high = ~0u;
             wfx[e] = v;
-            s += (unsigned long long)v;
-            f += (float)v;
+            add_seen(s, (unsigned long long)v, high);
         }
 #pragma unroll
-        for (int o = ROW / 2; o; o >>= 1) {
-            s += __shfl_xor_sync(FULL_MASK, s, o);
-            f += __shfl_xor_sync(FULL_MASK, f, o);
-        }
+        for (int o = ROW / 2; o; o >>= 1) add_seen(s, __shfl_xor_sync(FULL_MASK, s, o), high);
         if (lane == 0 && u < n) {
             k[u] = (i64)s;
             logk[u] = s ? log2f((float)(i64)s) : 0.0f;
-            tot += s;
-            tot_f += f;
+            add_seen(tot, s, high);
             kmax = max(kmax, s);
         }
     }
-    if (mask) atomicOr(&ps->range, mask);
-    add_totals(tot, tot_f, kmax, ps);
+    add_totals(tot, kmax, high, ps);
 }
 
 int first_category(u32 mask) {
@@ -244,7 +237,7 @@ int first_category(u32 mask) {
 int graph_prepare(i64 n, i64 nnz, const i64 *rp, const i32 *col, const float *w, i64 *wfx, i64 *k, float *logk,
                   DevGraph *g, cudaStream_t st) {
     PrepState *ps = nullptr;
-    const PrepState init{0u, 0u, 0u, INT32_MAX, 0ull, 0.0, 0ull, 0ull};
+    const PrepState init{0u, 0u, 0u, INT32_MAX, 0ull, 0ull, 0ull};
     MSCD_CUDA(cudaMallocAsync((void **)&ps, sizeof(PrepState), st));
     int rc = MSCD_OK;
     PrepState h{};
@@ -269,7 +262,6 @@ int graph_prepare(i64 n, i64 nnz, const i64 *rp, const i32 *col, const float *w,
         u32 found = h.rows | h.mask;
         if (!found && h.below) found = CAT_NOTSYM;
         if ((rc = first_category(found | h.range))) break;
-        if (h.total_d >= 0x1p63 || h.total >= (1ull << 62)) { rc = MSCD_ERANGE; break; }
         g->n = n;
         g->nnz = nnz;
         g->rp = rp;
