@@ -63,11 +63,12 @@
 // What bounds the kernel is the chain of dependent steps of an addition
 // (argmax, the top's row, its neighbours' buckets, their slots) and the
 // instructions issued along it, not bytes.  Hence the split into a short loop
-// that stays in registers (pop the top, test it, scan its row) and
-// out-of-line functions for everything else (next_row: initial members, the
-// start of a round, bulk rejections, prune passes), which take the unit over
-// in shared memory: with all of it inlined the kernel wanted 160 registers,
-// spilled in the loop at 16 units per SM and waited for instructions.  Growth
+// (pop the top, test it, scan its row) and out-of-line functions for everything
+// else (next_row: initial members, the start of a round, bulk rejections, prune
+// passes), which take the unit over in shared memory: with all of it inlined the
+// kernel wanted 160 registers, spilled in the loop at 16 units per SM and waited
+// for instructions.  With 128 registers nothing is spilled now; with the 80 of
+// the arena classes up to 32,768 slots 116 to 152 bytes a thread are.  Growth
 // of the 1-of-8 run of the 100,000-node graph (250,000 units, the shared class
 // and the 8,192-slot one): 48 + 237 ms before, 26 + 139 now; of the 1-of-80 run
 // of the weighted 1M-node graph 41 + 461, now 28 + 272.
@@ -97,8 +98,8 @@ __device__ __forceinline__ float unord(int o) { return __int_as_float(o >= 0 ? o
 constexpr int ORD_NEG_INF = (int)(0xff800000u ^ 0x7fffffffu);
 constexpr float NEG_INF = -__builtin_huge_valf();
 
-// __log2f for arguments that are 0 or at least 1 (the same value: only
-// denormal arguments differ, which that handles with three more instructions).
+// __log2f for arguments that are 0 or at least 1: with .ftz, lg2 takes subnormal
+// arguments for 0, and there are none.
 __device__ __forceinline__ float log2_int(float x) {
     float y;
     asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));

@@ -23,12 +23,13 @@
 //     subadditive), and h(P11) = 0, so the admission test fails.
 //     Either side of such a pair may be the small one, so the partners
 //     listed for this test are the B communities with 2(|B| + a) > n, a the
-//     largest active A community of the part; each A community walks its
-//     part's list in descending size and stops at the first B too small.
+//     largest active A community of the part; each A community with
+//     2(|A| + b) > n, b the largest listed, goes through its part's list and
+//     takes those that are large enough.
 // The intersections of the sharing pairs are counted by a warp per community:
 // it takes 32 of its members at a time, lays their lists of partner
-// communities end to end (the lanes then load 32 entries of several lists at
-// once, and the next ones while these are counted) and counts in a
+// communities end to end where they are short (the lanes then load 32 entries of
+// several lists at once, and the next ones while these are counted) and counts in a
 // shared-memory hash; a community with many members' lists to walk, or that
 // meets too many partners, is done by a whole CTA with a larger shared-memory
 // table, and beyond that with a global-memory table of its own.  A listed

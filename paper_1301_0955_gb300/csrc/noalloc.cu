@@ -161,7 +161,7 @@ extern "C" int mscd_grow_noalloc(mscd_ctx *ctx, int32_t graph_id, const double *
     // Shared-memory classes first (shared memory is no allocation, and they keep
     // every SM busy, which the scratch's 200-300 arenas cannot); what outgrows
     // them runs in the arenas.  2,048 seeds at 4 scales of a 100,000-node graph:
-    // 18.5 ms in the arenas alone, 9.2 now.
+    // 18.5 ms in the arenas alone, 7.8 now.
     int sms = 1;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     i64 full = 32;
