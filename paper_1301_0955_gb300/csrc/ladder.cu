@@ -107,9 +107,9 @@ int make_ladder(const DevGraph &G, i64 max_part_n, const mscd_params &p, std::ve
         // that touch more than 8,192 nodes take 34 ms at 16,384 slots, 41 at 32,768
         // and 52 at 65,536.  Among the wide ones a state of 65,536 weighted slots is
         // 2.4 MB, of 131,072 4.8: long lists need the smaller one, as the arena holds
-        // 1,807 or 903 units (22,112 units that touch up to 140,000 nodes of a weighted
-        // 300,000-node graph: 9.1 s with it, 13.3 without), and short ones skip it
-        // (see grow_units).
+        // 1,807 or 903 units (22,112 units of a weighted 300,000-node graph that touch
+        // more than 16,384 nodes, 94 of them more than 65,536: 9.2 s with it, 13.3
+        // without), and short ones skip it (see grow_units).
         i64 next = cg * 8;
         for (const i64 v : KEPT_SLOTS)
             if (v > cg && v < next) {
