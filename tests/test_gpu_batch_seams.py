@@ -48,11 +48,13 @@ def test_stability_in_several_chunks(mscd_mod):
     assert len(set(want)) > 5  # the scales differ, on both sides of the seams
     # room for two scales (and the table of terms), not for eleven
     torch.cuda.synchronize()
-    hold = torch.empty(torch.cuda.mem_get_info()[0] - (500 << 20), dtype=torch.uint8, device="cuda")
+    hold, left = [], 500 << 20
     try:
+        while (free := torch.cuda.mem_get_info()[0]) > left + (64 << 20):
+            hold.append(torch.empty(min(free - left, 16 << 30), dtype=torch.uint8, device="cuda"))
         again, nmi2 = run()
     finally:
-        del hold
+        hold.clear()
         torch.cuda.empty_cache()
     assert np.array_equal(nmi2, want)
     for a, b in zip(covers, again):
